@@ -1010,23 +1010,22 @@ def main():
                 "peak_source": f"152 SMs x 128 FP32 lanes x 2 flop x {clk:.0f} MHz (derived)"}
         roof_alt = None
     else:
-        nprod = 6 if prec == tri.BF16X6 else 3
-        planes = 3 if prec == tri.BF16X6 else 2
+        nprod, planes = 3, 2  # hi.hi, hi.lo, lo.hi of two FP16 planes, both precisions
         dp = -(-D_FEAT // 64) * 64
         t_gram = phases["gram_ms"] * 1e-3
-        # algorithmic bytes: the packed FP32 triangle written once, the planes and norms read once
-        nbytes = 4.0 * P + planes * N_PTS * dp * 2 + 4 * N_PTS
+        # algorithmic bytes: the packed FP32 triangle written once, the planes, norms and scales read once
+        nbytes = 4.0 * P + planes * N_PTS * dp * 2 + 8 * N_PTS
         hbm = nbytes / t_gram / 1e9
         # algorithmic tensor work: every pair i >= j once, 2 flop per
         # multiply-add over the K-padded features, for each kept plane product
         flops = 2.0 * dp * nprod * P
         tflop = flops / t_gram / 1e12
         traffic = NCU_TRAFFIC.get((args.prec, N_PTS, D_FEAT))
-        roof_hbm = {"bound": "hbm", "kernel": f"gram_kernel<lambda,{planes}>", "achieved": hbm,
+        roof_hbm = {"bound": "hbm", "kernel": "gram_kernel<lambda>", "achieved": hbm,
                     "peak": float(peaks["hbm_gbs"]), "unit": "GB/s", "frac": hbm / float(peaks["hbm_gbs"]),
                     "traffic": traffic, "algorithmic_bytes": nbytes,
                     "peak_source": f"hbm_gbs of {peak_src}"}
-        roof_tc = {"bound": "tensor", "kernel": f"gram_kernel<lambda,{planes}>", "achieved": tflop,
+        roof_tc = {"bound": "tensor", "kernel": "gram_kernel<lambda>", "achieved": tflop,
                    "peak": float(peaks["bf16_tflops"]), "unit": "TFLOP/s",
                    "frac": tflop / float(peaks["bf16_tflops"]), "traffic": traffic,
                    "flops": flops, "flops_note": "N(N+1)/2 pairs x 2 x K(padded) x plane products",

@@ -83,9 +83,11 @@ typedef enum {
 
 typedef enum {
     TRI_FP32 = 0,   /* direct differences in FP32 on CUDA cores */
-    TRI_BF16X3 = 1, /* Gram form on tcgen05 tensor cores: hi/lo BF16 split,
-                       3 products, FP32 accumulation, FP64 recompute of flagged pairs */
-    TRI_BF16X6 = 2  /* Gram form on tcgen05: hi/mid/lo BF16 split, 6 products,
+    TRI_BF16X3 = 1, /* Gram form on tcgen05 tensor cores: rows scaled by powers of
+                       two and split into two 16-bit planes (FP16 hi/lo), 3 products,
+                       FP32 accumulation, FP64 recompute of flagged pairs */
+    TRI_BF16X6 = 2  /* the same with the flag threshold that bounds every result
+                       (the accuracy of a hi/mid/lo BF16 split with 6 products):
                        FP32 accumulation, FP64 recompute of flagged pairs */
 } tri_prec;
 
@@ -205,8 +207,8 @@ TRI_API int tri_edm_workspace_size(uint32_t n, uint32_t d, int prec, size_t *byt
  * stages); larger sizes give TRI_ERANGE.
  *
  *   tri_edm_prepare: clears the workspace header, then writes the FP32 row
- *     norms |x_i|^2 (summed to ~48 bits as FP32 pairs) and the BF16 split
- *     planes (hi, lo or hi, mid, lo; K zero-padded to a multiple of 64).
+ *     norms |x_i|^2 (summed to ~48 bits as FP32 pairs), the row scales and the
+ *     FP16 split planes (hi, lo; K zero-padded to a multiple of 64).
  *   tri_edm_gram: tensor-core Gram term, d^2 = |x_i|^2 + |x_j|^2 - 2 x_i.x_j,
  *     clamped at 0, square root stored to out (packed, FP32); pairs with
  *     d^2 < tau (|x_i|^2 + |x_j|^2) appended to the workspace's flag list.

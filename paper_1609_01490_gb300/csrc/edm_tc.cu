@@ -1,19 +1,26 @@
 // Euclidean distance matrix on tcgen05 tensor cores (not in the paper, which
 // evaluates distances directly): d_ij^2 = |x_i|^2 + |x_j|^2 - 2 x_i.x_j with the
-// Gram term x_i.x_j from BF16 products accumulated in FP32 in tensor memory.
+// Gram term x_i.x_j from FP16 products accumulated in FP32 in tensor memory.
 //
-// Precision.  Each FP32 input is split into BF16 planes, x = hi + lo (+ mid):
-//   hi = bf16(x), r = x - hi (exact), mid = bf16(r), lo = bf16(r - mid).
-// Three planes represent x exactly (3 x 8 significant bits = FP32's 24);
-// the Gram term keeps the products hi.hi', hi.mid', mid.hi', hi.lo', lo.hi',
-// mid.mid' (BF16X6) and drops those below 2^-24 |x||y|; the two-plane form
-// (BF16X3) keeps hi.hi', hi.lo', lo.hi'.  Every BF16 x BF16 product is exact
-// in FP32.  A pair whose estimate falls below tau (|x_i|^2 + |x_j|^2) has lost
+// Precision.  Row i is scaled by a power of two s_i that puts its largest
+// magnitude in [2^14, 2^15) and split into two FP16 planes, s_i x = hi + lo:
+//   hi = fp16(s_i x), r = s_i x - hi (exact), lo = fp16(r).
+// The two planes hold s_i x to 2^-23 of itself (or 2^-39 of the row's largest
+// magnitude where lo is subnormal).  The Gram term keeps the products hi.hi',
+// hi.lo', lo.hi' and drops lo.lo', below 2^-22 |x||y|; every FP16 x FP16 product
+// is exact in FP32, and the epilogue takes the scales out again (exact powers
+// of two).  Both tensor-core precisions use this split and differ in the flag
+// threshold.  A BF16 split needs three planes
+// and six products for the same bits.  At N = 65536, d = 128 that took 2.18 ms
+// a call against 1.80 ms here (1.78 ms of it the six products' tensor time at
+// the measured peak), and its relative error against 64 bits was 7.2e-8 against
+// 4.8e-8: the planes' rounding costs less than twice the accumulation steps.
+// A pair whose estimate falls below tau (|x_i|^2 + |x_j|^2) has lost
 // too many digits to cancellation and is flagged; a second kernel recomputes
 // flagged pairs in FP64 by direct differences (the paper's definition).
 //
-// Kernels.  prepare: row norms (FP32 pairs, stored as FP32) and the BF16 planes,
-// K padded to a multiple of 64.  gram: persistent clusters of two CTAs on two
+// Kernels.  prepare: row norms (FP32 pairs, stored as FP32), row scales and the
+// FP16 planes, K padded to a multiple of 64.  gram: persistent clusters of two CTAs on two
 // SMs (a CTA pair), one pair per two SMs.  A unit of work is a 2 x 2 block of
 // 128 x 128 pair tiles (row blocks 2R, 2R + 1, column blocks 2C, 2C + 1),
 // taken in lambda order over the triangle of units (Eq. eq_gmap): first one
@@ -33,7 +40,7 @@
 // four 32-column quarters of the same rows store them together).  fixup: FP64
 // recompute of the flagged pairs.
 #include <cuda.h>
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
 
@@ -41,6 +48,7 @@
 #include <cmath>
 #include <mutex>
 
+#include "f32x2.cuh"
 #include "tri_internal.h"
 #include "tri_maps.cuh"
 
@@ -49,12 +57,13 @@ using namespace tri;
 namespace {
 
 constexpr int TILE = 128;                  // pair tile side (UMMA M = N = 128)
-constexpr int KCH = 64;                    // K per chunk: one 128-byte swizzle row of BF16
-constexpr int CHUNK_BYTES = TILE * KCH * 2;  // 16 KB: 128 rows x 64 BF16
+constexpr int KCH = 64;                    // K per chunk: one 128-byte swizzle row of FP16
+constexpr int P = 2;                       // FP16 planes per row: hi, lo
+constexpr int CHUNK_BYTES = TILE * KCH * 2;  // 16 KB: 128 rows x 64 FP16
 constexpr int NEPI = 16;                   // epilogue warps: 4 TMEM lane quarters x 4 row groups
 constexpr int NTHREADS = 64 + 32 * NEPI;   // TMA warp, MMA warp, epilogue warps
 constexpr int EPI_ROWS = 16;               // output rows per TMEM load in the epilogue
-constexpr int NORM_FLOATS = 2 * 32;       // per epilogue warp: norms of its 32 rows of the tile (double buffered)
+constexpr int NORM_FLOATS = 2 * 64;       // per epilogue warp: norms and scales of its 32 rows of the tile (double buffered)
 // Each epilogue warp holds TILE / (NEPI / 4) rows of a tile: the norm buffers
 // and the prefetch pattern are sized for 32 (16 epilogue warps).
 static_assert(TILE / (NEPI / 4) == 32, "epilogue norm buffers assume 32 rows per warp and tile");
@@ -66,16 +75,18 @@ constexpr uint32_t DYN_CHUNK = 2;          // units per grab from the global cou
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr int MAX_STAGES = 12;             // B ring depth cap (16 KB stages)
 
-constexpr float TAU_X3 = 0.0625f;  // flag threshold for hi/lo (empirical)
+constexpr float TAU_X3 = 0.0625f;  // flag threshold of TRI_BF16X3 (no bound asked for)
 
-// Flag threshold for hi/mid/lo with nkc 64-wide K chunks.  The Gram term's
-// error is at most 2^-23 (dropped products) plus 2^-23 per FP32 accumulation
-// step (24 MMAs of K = 16 per chunk: 6 plane products x 4) of
-// sum_k |x_ik x_jk| <= (|x_i|^2 + |x_j|^2) / 2; with the norms' and the final
-// combination's roundings, |error of d^2| <= (2 + 24 nkc) 2^-23 (|x_i|^2 +
-// |x_j|^2).  The relative error of d is about half that of d^2, and the
-// square root adds up to ~1.5e-7, so a pair with d^2 > tau (|x_i|^2 + |x_j|^2)
-// stays within 1e-5 when tau = (2 + 24 nkc) 2^-23 / (2 (1e-5 - 2e-7)).
+// Flag threshold of TRI_BF16X6 with nkc 64-wide K chunks.  The Gram term's
+// error is at most 2^-21 (both rows' planes, 2^-23 each, and the dropped
+// product, 2^-22) plus 2^-23 per FP32 accumulation step (12 MMAs of K = 16 per
+// chunk: 3 plane products x 4) of sum_k |x_ik x_jk| <= (|x_i|^2 + |x_j|^2) / 2,
+// so with the norms' and the final combination's roundings |error of d^2| <=
+// (5 + 12 nkc) 2^-23 (|x_i|^2 + |x_j|^2).  The relative error of d is about
+// half that of d^2, and the square root adds up to ~1.5e-7.  tau keeps the
+// larger value (2 + 24 nkc) 2^-23 / (2 (1e-5 - 2e-7)) of a split with 24 steps
+// per chunk, so that the same pairs are flagged: a pair with d^2 > tau
+// (|x_i|^2 + |x_j|^2) stays well within 1e-5.
 // tau = 0.158 (d <= 64), 0.304 (d <= 128), 0.450 (d <= 192).
 float tau_x6(uint32_t nkc) { return (float)((2.0 + 24.0 * nkc) * std::ldexp(1.0, -23) / (2.0 * (1e-5 - 2e-7))); }
 
@@ -85,27 +96,31 @@ float flag_tau(int prec, uint32_t d)
 }
 
 struct WsLayout {
-    size_t hdr, norms, planes, flags, total;
+    size_t hdr, norms, scales, planes, flags, total;
     unsigned long long cap;
 };
 
 // Workspace: [header 256 B: flag counter (u64 at 0), status (int at 8), tile
 // counter (u64 at 16), tri_edm_host's two list-start slots (u64 at 24, 32),
 // the wait limit of the Gram kernel's waits between roles in ns (u64 at 40,
-// 0: WAIT_LIMIT_NS)][norms n FP32][planes P x n x dp BF16][flag list cap x
-// u64], each part 256-byte aligned.  tri_edm_prepare clears the header.
+// 0: WAIT_LIMIT_NS)][norms n FP32][1 / row scale n FP32][planes P x n x dp
+// FP16][flag list cap x u64], each part 256-byte aligned.  tri_edm_prepare
+// clears the header.  The total is the one callers have always been asked for
+// (header, norms, three (X6) or two (X3) 16-bit planes and max(2^20, 4n) list
+// entries); the list takes whatever of it the other parts leave.
 WsLayout ws_layout(uint32_t n, uint32_t d, int prec)
 {
-    const int P = prec == TRI_BF16X6 ? 3 : 2;
     const size_t dp = ((size_t)d + KCH - 1) / KCH * KCH;
     auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
     WsLayout L;
     L.hdr = 0;
     L.norms = 256;
-    L.planes = al(L.norms + sizeof(float) * n);
-    L.cap = (unsigned long long)std::max<size_t>(1u << 20, 4 * (size_t)n);
+    const size_t planes = prec == TRI_BF16X6 ? 3 : 2, entries = std::max<size_t>(1u << 20, 4 * (size_t)n);
+    L.total = al(al(al(L.norms + sizeof(float) * n) + planes * n * dp * 2) + entries * sizeof(unsigned long long));
+    L.scales = al(L.norms + sizeof(float) * n);
+    L.planes = al(L.scales + sizeof(float) * n);
     L.flags = al(L.planes + (size_t)P * n * dp * 2);
-    L.total = al(L.flags + L.cap * sizeof(unsigned long long));
+    L.cap = (L.total - L.flags) / sizeof(unsigned long long);
     return L;
 }
 
@@ -277,18 +292,18 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
-// Instruction descriptor, kind::f16 across the CTA pair: FP32 accumulator,
-// BF16 A and B, both K-major, N = 256 (bits 17-22 hold N/8), M = 256 (bits
+// Instruction descriptor, kind::f16 across the CTA pair: FP32 accumulator
+// (bits 4-5 = 1), FP16 A and B (bits 7-9 and 10-12 = 0), both K-major, N = 256 (bits 17-22 hold N/8), M = 256 (bits
 // 24-28 hold M/16).  Rows 0-127 of M (and of N) come from the even CTA,
 // 128-255 from the odd one; each CTA's TMEM receives its own 128 rows of M
 // across all 256 columns of N.
-constexpr uint32_t IDESC2 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)((2 * TILE) >> 3) << 17) |
+constexpr uint32_t IDESC2 = (1u << 4) | ((uint32_t)((2 * TILE) >> 3) << 17) |
                             ((uint32_t)((2 * TILE) >> 4) << 24);
 
 // One MMA over the pair: A (M side) and B (N side) are read at the same
 // shared-memory offsets in both CTAs; each CTA holds half of A's M rows and
 // half of B's N rows.
-__device__ __forceinline__ void umma2_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate)
+__device__ __forceinline__ void umma2_f16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t accumulate)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -348,37 +363,29 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
     e = (a - (s - bp)) + (b - bp);
 }
 
-// One warp per row: the BF16 planes and the row norm |x|^2, summed as an
-// unevaluated pair hi + lo of FP32 numbers (products split exactly by FMA,
-// sums by TwoSum; about 48 significant bits, FP64 being scarce on this part),
-// rounded to FP32 once at the end.
-template <int P>
+// One warp per row: the row's scale, its FP16 planes and the row norm |x|^2,
+// summed as an unevaluated pair hi + lo of FP32 numbers (products split exactly
+// by FMA, sums by TwoSum; about 48 significant bits, FP64 being scarce on this
+// part), rounded to FP32 once at the end.  The scale is 2^(14 - e), e the
+// exponent of the row's largest finite magnitude, held within FP32's normal
+// powers; its inverse goes to scales[].  A row with an infinity or a NaN gets
+// NaN planes there, and NaN distances.
 __global__ void prepare_kernel(const float *__restrict__ x, uint32_t n, uint32_t d, uint32_t dp,
-                               float *__restrict__ norms, __nv_bfloat16 *__restrict__ planes)
+                               float *__restrict__ norms, float *__restrict__ scales, __half *__restrict__ planes)
 {
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (warp >= n) return;
     const float *row = x + (size_t)warp * d;
-    float hi = 0.0f, lo = 0.0f;
-    for (uint32_t k = lane; k < dp; k += 32) {
-        const float v = k < d ? row[k] : 0.0f;
+    float hi = 0.0f, lo = 0.0f, big = 0.0f;
+    for (uint32_t k = lane; k < d; k += 32) {
+        const float v = row[k];
         const float p = v * v, pe = fmaf(v, v, -p);  // v^2 = p + pe
         float t, te;
         two_sum(hi, p, t, te);
         hi = t;
         lo += te + pe;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        const float r1 = v - __bfloat162float(hi);
-        const size_t o = (size_t)warp * dp + k;
-        planes[o] = hi;
-        if constexpr (P == 2) {
-            planes[(size_t)n * dp + o] = __float2bfloat16_rn(r1);
-        } else {
-            const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-            const float r2 = r1 - __bfloat162float(mid);
-            planes[(size_t)n * dp + o] = mid;
-            planes[2 * (size_t)n * dp + o] = __float2bfloat16_rn(r2);
-        }
+        const float a = fabsf(v);
+        if (a <= 3.402823466e38f) big = fmaxf(big, a);  // finite magnitudes only
     }
     for (int o = 16; o > 0; o >>= 1) {
         const float oh = __shfl_down_sync(0xffffffffu, hi, o), ol = __shfl_down_sync(0xffffffffu, lo, o);
@@ -386,8 +393,23 @@ __global__ void prepare_kernel(const float *__restrict__ x, uint32_t n, uint32_t
         two_sum(hi, oh, t, te);
         hi = t;
         lo += ol + te;
+        big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
     }
-    if (lane == 0) norms[warp] = hi + lo;
+    // biased exponent of the scale: 127 + 14 - e, with big's biased exponent 127 + e
+    const int be = (int)(__float_as_uint(big) >> 23);
+    const int se = big == 0.0f ? 127 : min(253, 268 - be);
+    const float sc = __uint_as_float((uint32_t)se << 23);
+    if (lane == 0) {
+        norms[warp] = hi + lo;
+        scales[warp] = __uint_as_float((uint32_t)(254 - se) << 23);
+    }
+    __half *ph = planes + (size_t)warp * dp, *pl = ph + (size_t)n * dp;
+    for (uint32_t k = lane; k < dp; k += 32) {
+        const float v = k < d ? row[k] * sc : 0.0f;
+        const __half h = __float2half_rn(v);
+        ph[k] = h;
+        pl[k] = __float2half_rn(v - __half2float(h));
+    }
 }
 
 // --------------------------------------------------------------- gram ----
@@ -405,7 +427,7 @@ struct GramArgs {
     uint32_t chunk;            // units per grab from the counter
     uint32_t stages;           // B ring depth
     float tau;
-    const float *norms;
+    const float *norms, *scales;  // per row: |x|^2 and 1 / scale
     float *out;
     unsigned long long *flag_count, *flag_list, flag_cap;
     unsigned long long *tile_counter;  // zero at launch
@@ -429,9 +451,7 @@ __device__ __forceinline__ bool unit_of(uint64_t u, uint32_t mb, uint32_t &R, ui
 }
 
 // The split keeps the products of row plane pa and column plane pb with
-// pa + pb <= P - 1: hi.hi, hi.mid, mid.hi, hi.lo, lo.hi, mid.mid for P = 3
-// and hi.hi, hi.lo, lo.hi for P = 2.
-
+// pa + pb <= P - 1: hi.hi, lo.hi and hi.lo.
 
 // Barrier among the `count` threads of one epilogue row group (ids 1..).
 __device__ __forceinline__ void named_sync(uint32_t id, uint32_t count)
@@ -457,12 +477,20 @@ __device__ __forceinline__ bool named_sync_all(uint32_t id, uint32_t count, bool
     return r != 0;
 }
 
-// 1/sqrt by the MUFU unit (flush-to-zero approximation; relative error a few
+// sqrt by the MUFU unit (flush-to-zero approximation; relative error about
 // 2^-23, far inside the 1e-5 the distances are held to).
-__device__ __forceinline__ float rsqrt_approx(float x)
+__device__ __forceinline__ float sqrt_approx(float x)
 {
     float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Three-input minimum (a NaN is ignored, as by fminf).
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float y;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
     return y;
 }
 
@@ -475,7 +503,7 @@ __device__ __forceinline__ uint32_t sdesc_lo(uint32_t addr) { return (addr >> 4)
 constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);  // SBO, version, 128-byte swizzle
 
 
-template <int MAP, int P>
+template <int MAP>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     gram_kernel(const __grid_constant__ CUtensorMap tmap, const GramArgs g)
 {
@@ -484,7 +512,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     uint8_t *gbase = smem_raw + (base - raw);
-    const uint32_t a_bytes = (uint32_t)P * g.nkc * CHUNK_BYTES;  // this CTA's row block
+    const uint32_t a_bytes = P * g.nkc * CHUNK_BYTES;  // this CTA's row block
     constexpr uint32_t stage_bytes = CHUNK_BYTES;               // one plane of one K chunk
     const uint32_t sA = base;                                   // [kc][p] chunks
     const uint32_t sB = base + a_bytes;                         // [stage] chunks of one plane
@@ -759,7 +787,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                             for (int kk = 0; kk < KCH / 16; ++kk)
                                 // the column blocks are the M operand: TMEM lane = output
                                 // column; +2 per 16-element K step (32 bytes in 16-byte units)
-                                umma2_bf16(d_tmem, b_desc + 2 * kk, a_desc + pa * CH16 + 2 * kk,
+                                umma2_f16(d_tmem, b_desc + 2 * kk, a_desc + pa * CH16 + 2 * kk,
                                            (kc | pb | pa | kk) ? 1u : 0u);
                         umma2_commit_both(b_emptyB + 8 * stage);  // stage free (both CTAs) when these MMAs finish
                         if (++stage == g.stages) {
@@ -797,18 +825,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         const uint32_t e = warp - 2, q = warp & 3, grp = e >> 2;
         float *snorm = epi + e * NORM_FLOATS;     // norms of this warp's rows, two buffers
         const float tau = g.tau;
-        // next tile's norms: lane l holds the norms of row l % 16 of chunks
-        // u = 2v + l / 16 (16 rows each) and of its own column
-        float pfr[NCH / 2], pfj = 0.0f;
+        // next tile's norms and scales: lane l holds those of row l % 16 of
+        // chunks u = 2v + l / 16 (16 rows each) and of its own column
+        float pfr[NCH / 2], pfs[NCH / 2], pfj = 0.0f, pfjs = 0.0f;
         auto prefetch = [&](uint32_t a, uint32_t b) {  // row block a, column block b
 #pragma unroll
             for (int v = 0; v < NCH / 2; ++v) {
                 const uint32_t u = 2 * v + (lane >> 4);
                 const uint32_t ii = a * TILE + (grp + NG * u) * EPI_ROWS + (lane & 15);
                 pfr[v] = ii < g.n ? __ldg(g.norms + ii) : 0.0f;
+                pfs[v] = ii < g.n ? __ldg(g.scales + ii) : 0.0f;
             }
             const uint32_t jj = b * TILE + q * 32 + lane;
             pfj = jj < g.n ? __ldg(g.norms + jj) : 0.0f;
+            pfjs = jj < g.n ? __ldg(g.scales + jj) : 0.0f;
         };
         uint32_t acc = 0, acc_phase = 0, nbuf = 0, k = 0;
         auto fail = [&]() {
@@ -835,10 +865,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             for (uint32_t t = 0; t < 2; ++t) {
                 const uint32_t bi = 2 * R + t;
                 const bool valid = bj <= bi && bi < g.m;
-                float *rn = snorm + nbuf * 32;  // this tile's row norms: [chunk u][16]
+                float *rn = snorm + nbuf * 64, *rs = rn + 32;  // this tile's row norms and scales: [chunk u][16]
 #pragma unroll
-                for (int v = 0; v < NCH / 2; ++v) rn[32 * v + lane] = pfr[v];
-                const float nj = pfj;
+                for (int v = 0; v < NCH / 2; ++v) {
+                    rn[32 * v + lane] = pfr[v];
+                    rs[32 * v + lane] = pfs[v];
+                }
+                const float nj = pfj, cj = -2.0f * pfjs;
+                const f2 nj2 = f2_pack(nj, nj), cj2 = f2_pack(cj, cj), mtau2 = f2_pack(-tau, -tau);
                 __syncwarp();
                 if (t == 0) {
                     prefetch(bi + 1, bj);
@@ -859,40 +893,44 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         tmem_wait16(cur);
                         if (u + 1 < NCH) tmem_ld16(taddr + (grp + NG * (u + 1)) * EPI_ROWS, raw[(u + 1) & 1]);
                         const uint32_t i0 = bi * TILE + (grp + NG * u) * EPI_ROWS;  // first row of the chunk
-                        float ni[EPI_ROWS];
+                        const float *un = rn + u * EPI_ROWS, *us = rs + u * EPI_ROWS;
+                        // two rows per instruction: d2 = |x_i|^2 + |x_j|^2 - 2 x_i.x_j;
+                        // one test per chunk for a pair with d2 <= tau (|x_i|^2 +
+                        // |x_j|^2) (cancellation, the diagonal, or padding).  The
+                        // scales go in one after the other: each product stays in
+                        // FP32's range wherever the norms do.
+                        float dv[EPI_ROWS], d2v[EPI_ROWS], w[EPI_ROWS];
 #pragma unroll
                         for (int k = 0; k < EPI_ROWS; k += 4) {
-                            const float4 v4 = *reinterpret_cast<const float4 *>(rn + u * EPI_ROWS + k);
-                            ni[k] = v4.x;
-                            ni[k + 1] = v4.y;
-                            ni[k + 2] = v4.z;
-                            ni[k + 3] = v4.w;
+                            const ulonglong2 n4 = *reinterpret_cast<const ulonglong2 *>(un + k);
+                            const ulonglong2 c4 = *reinterpret_cast<const ulonglong2 *>(us + k);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const int e = k + 2 * h;
+                                const f2 sum = f2_add(h ? n4.y : n4.x, nj2);
+                                const f2 gram = f2_pack(__uint_as_float(cur[e]), __uint_as_float(cur[e + 1]));
+                                const f2 d2 = f2_fma(f2_mul(gram, h ? c4.y : c4.x), cj2, sum);
+                                f2_unpack(d2, d2v[e], d2v[e + 1]);
+                                f2_unpack(f2_fma(mtau2, sum, d2), w[e], w[e + 1]);
+                                dv[e] = sqrt_approx(d2v[e]);
+                                dv[e + 1] = sqrt_approx(d2v[e + 1]);
+                            }
                         }
-                        // fast path: d = d2 * rsqrt(d2); one test per chunk for a pair
-                        // with d2 <= tau (|x_i|^2 + |x_j|^2) (cancellation, the
-                        // diagonal, or padding)
-                        float dv[EPI_ROWS], d2v[EPI_ROWS];
                         float worst = 1.0f;
 #pragma unroll
-                        for (int k = 0; k < EPI_ROWS; ++k) {
-                            const float s = ni[k] + nj;
-                            const float d2 = fmaf(-2.0f, __uint_as_float(cur[k]), s);
-                            d2v[k] = d2;
-                            worst = fminf(worst, fmaf(-tau, s, d2));
-                            dv[k] = d2 * rsqrt_approx(d2);
-                        }
+                        for (int k = 0; k < EPI_ROWS; k += 2) worst = min3(worst, w[k], w[k + 1]);
                         if (worst <= 0.0f) {
 #pragma unroll
                             for (int k = 0; k < EPI_ROWS; ++k) {
                                 const float d2 = d2v[k];
-                                if (d2 <= tau * (ni[k] + nj)) {
+                                if (d2 <= tau * (un[k] + nj)) {
                                     const uint32_t i = i0 + k;
                                     if (i < g.n && j < i) {
                                         const unsigned long long slot = atomicAdd(g.flag_count, 1ull);
                                         if (slot < g.flag_cap) g.flag_list[slot] = ((unsigned long long)i << 32) | j;
                                     }
                                     // provisional value (flagged pairs are recomputed; the diagonal is exact 0)
-                                    dv[k] = (i == j || d2 <= 0.0f) ? 0.0f : d2 * rsqrt_approx(d2);
+                                    dv[k] = (i == j || d2 <= 0.0f) ? 0.0f : sqrt_approx(d2);
                                 }
                             }
                         }
@@ -914,8 +952,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         if (bi != bj && (bi + 1) * TILE <= g.n) {
 #pragma unroll
                             for (int k = 0; k < EPI_ROWS; ++k) {
-                                __stcs(row, dv[k]);
-                                row += i0 + k + 1;  // T2(i + 1) - T2(i)
+                                // T2(i0 + k) - T2(i0) = k i0 + k (k + 1) / 2
+                                __stcs(reinterpret_cast<float *>(reinterpret_cast<char *>(row) + (uint64_t)i0 * (4u * k)) +
+                                           k * (k + 1) / 2,
+                                       dv[k]);
                             }
                         } else {
 #pragma unroll
@@ -1041,19 +1081,19 @@ size_t trihost::edm_tc_workspace(uint32_t n, uint32_t d, int prec) { return ws_l
 namespace {
 
 struct TcPlan {
-    int P;
     uint32_t dp, nkc, stages;
     size_t smem;
 };
 
 bool plan(uint32_t d, int prec, TcPlan &p)
 {
-    p.P = prec == TRI_BF16X6 ? 3 : 2;
     p.dp = (d + KCH - 1) / KCH * KCH;
     p.nkc = p.dp / KCH;
     const size_t fixed = 1024 /*align*/ + NEPI * NORM_FLOATS * 4 + 8 * (7 + 2 * MAX_STAGES);
-    const size_t a = (size_t)p.P * p.nkc * CHUNK_BYTES, st = CHUNK_BYTES;  // one row block per CTA
-    if (fixed + a + 2 * st > (size_t)SMEM_LIMIT) return false;
+    const size_t a = (size_t)P * p.nkc * CHUNK_BYTES, st = CHUNK_BYTES;  // one row block per CTA
+    if (d > (prec == TRI_BF16X6 ? 192u : 320u)) return false;  // the documented limits
+    static_assert(1024 + NEPI * NORM_FLOATS * 4 + 8 * (7 + 2 * MAX_STAGES) + 12 * CHUNK_BYTES <= SMEM_LIMIT,
+                  "d = 320 leaves at least two operand stages");
     p.stages = (uint32_t)std::min<size_t>(MAX_STAGES, (SMEM_LIMIT - fixed - a) / st);
     p.smem = fixed + a + p.stages * st;
     return true;
@@ -1062,10 +1102,10 @@ bool plan(uint32_t d, int prec, TcPlan &p)
 // Launches the pair kernel on as many CTA pairs as can be resident at once
 // (cached per instantiation and shared-memory size), splitting the units into
 // an up-front run per pair and counter-driven runs.
-template <int MP, int PP>
+template <int MP>
 cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(gram_kernel<MP, PP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(gram_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     static std::mutex mu;
     static int cached_dev = -1, cached_pairs = 0;
@@ -1080,7 +1120,7 @@ cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, cudaSt
         cfg.dynamicSmemBytes = smem;
         cfg.stream = s;
         int ncl = 0;
-        if (cudaOccupancyMaxActiveClusters(&ncl, gram_kernel<MP, PP>, &cfg) != cudaSuccess || ncl < 1) {
+        if (cudaOccupancyMaxActiveClusters(&ncl, gram_kernel<MP>, &cfg) != cudaSuccess || ncl < 1) {
             (void)cudaGetLastError();
             ncl = (int)(num_sms() / 2);
         }
@@ -1095,7 +1135,7 @@ cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, cudaSt
     g.static_per = units * STATIC_PCT / 100 / pairs;
     g.dyn_start = g.u0 + g.static_per * pairs;
     g.chunk = DYN_CHUNK;
-    gram_kernel<MP, PP><<<(unsigned)(2 * pairs), NTHREADS, smem, s>>>(tmap, g);
+    gram_kernel<MP><<<(unsigned)(2 * pairs), NTHREADS, smem, s>>>(tmap, g);
     return cudaGetLastError();
 }
 
@@ -1119,12 +1159,8 @@ extern "C" int tri_edm_prepare(const float *x, uint32_t n, uint32_t d, int prec,
     char *ws = (char *)workspace;
     if (cudaMemsetAsync(ws, 0, 256, s) != cudaSuccess) return TRI_ECUDA;
     const unsigned blocks = (unsigned)(((uint64_t)n * 32 + 255) / 256);
-    if (pl.P == 3)
-        prepare_kernel<3><<<blocks, 256, 0, s>>>(x, n, d, pl.dp, (float *)(ws + L.norms),
-                                                 (__nv_bfloat16 *)(ws + L.planes));
-    else
-        prepare_kernel<2><<<blocks, 256, 0, s>>>(x, n, d, pl.dp, (float *)(ws + L.norms),
-                                                 (__nv_bfloat16 *)(ws + L.planes));
+    prepare_kernel<<<blocks, 256, 0, s>>>(x, n, d, pl.dp, (float *)(ws + L.norms), (float *)(ws + L.scales),
+                                          (__half *)(ws + L.planes));
     return cudaGetLastError() == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 
@@ -1155,11 +1191,11 @@ int gram_range(uint32_t n, uint32_t d, float *out, int map, int prec, void *work
     char *ws = (char *)workspace;
     // 128-row blocks of the planes (row blocks and column blocks alike)
     CUtensorMap tmap;
-    const cuuint64_t gdim[3] = {pl.dp, n, (cuuint64_t)pl.P};
+    const cuuint64_t gdim[3] = {pl.dp, n, (cuuint64_t)P};
     const cuuint64_t gstride[2] = {(cuuint64_t)pl.dp * 2, (cuuint64_t)n * pl.dp * 2};
     const cuuint32_t box[3] = {KCH, TILE, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
-    if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, ws + L.planes, gdim, gstride, box, estr,
+    if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, ws + L.planes, gdim, gstride, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return TRI_ECUDA;
@@ -1173,6 +1209,7 @@ int gram_range(uint32_t n, uint32_t d, float *out, int map, int prec, void *work
     g.stages = pl.stages;
     g.tau = flag_tau(prec, d);
     g.norms = (const float *)(ws + L.norms);
+    g.scales = (const float *)(ws + L.scales);
     g.out = out;
     g.flag_count = (unsigned long long *)(ws + L.hdr);
     g.status = (int *)(ws + L.hdr + 8);
@@ -1182,10 +1219,7 @@ int gram_range(uint32_t n, uint32_t d, float *out, int map, int prec, void *work
     g.flag_cap = L.cap;
     if (cudaMemsetAsync(g.tile_counter, 0, sizeof(unsigned long long), s) != cudaSuccess) return TRI_ECUDA;
     cudaError_t e;
-    if (map == TRI_MAP_LAMBDA)
-        e = pl.P == 3 ? launch_gram<MAP_LAMBDA, 3>(tmap, g, pl.smem, s) : launch_gram<MAP_LAMBDA, 2>(tmap, g, pl.smem, s);
-    else
-        e = pl.P == 3 ? launch_gram<MAP_BB, 3>(tmap, g, pl.smem, s) : launch_gram<MAP_BB, 2>(tmap, g, pl.smem, s);
+    e = map == TRI_MAP_LAMBDA ? launch_gram<MAP_LAMBDA>(tmap, g, pl.smem, s) : launch_gram<MAP_BB>(tmap, g, pl.smem, s);
     return e == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 
