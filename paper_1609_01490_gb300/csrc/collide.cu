@@ -8,6 +8,7 @@
 // s = (c_i0 - c_j0)^2 + (c_i1 - c_j1)^2 + ..., each step a separate FP32
 // operation rounded to nearest (no fused multiply-add), so the decisions are
 // exactly those of any other implementation that takes the same steps.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "f32x2.cuh"
@@ -70,13 +71,13 @@ __device__ __forceinline__ void record(const CollideOut &o, uint32_t i, uint32_t
 // test of its one pair.  Not inlined: every block map calls the same body.
 template <int RHO, int R, int DIM>
 __device__ __noinline__ void collide_tile(const float *__restrict__ c, const float *__restrict__ rad, uint32_t n,
-                                          uint32_t bi, uint32_t bj, CollideOut o)
+                                          uint32_t bi, uint32_t bj, CollideOut o, int tx, int ty)
 {
     constexpr int S = RHO * R;
     constexpr int RC = R == 1 ? 1 : R / 2;
     __shared__ f2 si[DIM + 1][S];                       // rows, duplicated
     __shared__ __align__(8) float sj[DIM + 1][S + 2];   // columns
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * RHO + tx;
+    const int tid = ty * RHO + tx;
     const uint64_t i0 = (uint64_t)bi * S, j0 = (uint64_t)bj * S;
     const float inf = __int_as_float(0x7f800000);
     // coalesced staging of S consecutive spheres: centres (S DIM floats), then radii
@@ -157,6 +158,321 @@ __device__ __noinline__ void collide_tile(const float *__restrict__ c, const flo
     }
 }
 
+// ------------------------------------------------- tensor-core filter ----
+// The library's own tile (reg = 0, 2-D and 3-D): FP16 tensor cores rule out the
+// pairs that surely do not touch, and the few others take the exact test.
+//
+// With X = sigma (c - c0), R = sigma r (c0 and the power of two sigma chosen per
+// block so that every |X_k|, |R| < 16),
+//   sigma^2 (q - s) / 2 = u_i + u_j + R_i R_j + X_i . X_j,  u = (R^2 - |X|^2) / 2,
+// is one inner product of 16 terms: X and R in two FP16 parts each (hi.hi',
+// hi.lo', lo.hi' of up to four coordinates) and u in two.  Its error is below
+// 2^-8: parts 2^-13, dropped lo.lo' 2^-14, u 2^-13, accumulation of terms up to
+// 1792 with at least 23 fraction bits kept 2^-9, rounding of c - c0 and of the
+// exact test's own operations 2^-11.  u carries 2^-9 extra per sphere, so a
+// negative value proves s > q as the exact test computes it.  A sphere with an
+// infinite or NaN coordinate, and every sphere of a block whose extent lies
+// outside [2^-50, 2^60] (where the exact test's squares may overflow or
+// vanish), gets u = 30000 and X = R = 0: its pairs always take the exact test.
+// Padding past n gets u = -30000.
+//
+// mma.sync m16n8k16 leaves each thread its results in registers, so the test of
+// 512 pairs per warp is 4 instructions on the tensor core, 8 three-input ANDs
+// and a vote, against about 50 packed FP32 instructions.
+// 65,536 spheres in 3-D take 229 us against 970 with the packed FP32 tile,
+// 9001 in 2-D 21 against 48.  The tensor core bounds it (one m16n8k16 per SM
+// takes 1.04 ns: 115 us), then the staging of each block's spheres.
+// The margin is 3e-5 of the block's squared extent, so it flags few pairs unless
+// most spheres crowd into a small part of that extent (or meet many others):
+// each warp counts the flags of its first 512 pairs, and a block that finds more
+// than 1 in 128 runs the packed FP32 tile instead (not where values are infinite
+// or squares may overflow or vanish: that tile's sign test and packed arithmetic
+// are not exact there, the one-pair test is).  On a line (1-D) the margin
+// alone flags 1 in 180 pairs (0.63 against 0.59 ms): those keep the FP32 tile.
+constexpr int MMA_THREADS = 256;
+#ifndef MMA_BLOCKS
+#define MMA_BLOCKS 4
+#endif
+constexpr unsigned FULL = 0xFFFFFFFFu;
+
+__device__ __forceinline__ float redux_min(float v)
+{
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float redux_max(float v)
+{
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// two floats rounded to FP16, a in the low half
+__device__ __forceinline__ uint32_t half2_bits(float a, float b)
+{
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&h);
+}
+
+__device__ __forceinline__ float2 half2_floats(uint32_t v)
+{
+    return __half22float2(*reinterpret_cast<const __half2 *>(&v));
+}
+
+// d (16 x 8, FP32) = a (16 x 16) b (16 x 8), FP16 operands
+__device__ __forceinline__ void mma_16x8x16(const uint2 a0, const uint2 a1, const uint2 b, uint32_t (&d)[4])
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, "
+        "%10, %10};"
+        : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+        : "r"(a0.x), "r"(a1.x), "r"(a0.y), "r"(a1.y), "r"(b.x), "r"(b.y), "f"(0.0f));
+}
+
+// One S x S tile by 8 warps: S / 64 row groups of 64 rows (four 16-row operands
+// kept in registers), the columns split among the warps that share one.
+template <int S, int DIM>
+__device__ __noinline__ void collide_tile_mma(const float *__restrict__ c, const float *__restrict__ rad, uint32_t n,
+                                              uint32_t bi, uint32_t bj, CollideOut o)
+{
+    constexpr int NT = MMA_THREADS, NW = NT / 32, PER = 2 * S / NT;  // spheres staged per thread
+    static_assert(S % 64 == 0 && S / 64 <= NW && PER >= 1, "row groups of 64 rows");
+    extern __shared__ __align__(16) unsigned char mma_smem[];
+    // operand records (16 halves) of the S rows and S columns, then the spheres themselves
+    uint4 *rec = reinterpret_cast<uint4 *>(mma_smem);
+    float4 *pos = reinterpret_cast<float4 *>(mma_smem + 2 * S * 32);
+    __shared__ float s_red[NW][2 * DIM + 1];
+    __shared__ uint32_t s_flags[NW];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint64_t i0 = (uint64_t)bi * S, j0 = (uint64_t)bj * S;
+    const float inf = __int_as_float(0x7f800000);
+
+    // sphere e of the tile: e < S row i0 + e, else column j0 + e - S
+    float v[PER][DIM + 1];
+    bool live[PER], finite[PER];
+    float lo[DIM], hi[DIM], rmax = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        lo[k] = inf;
+        hi[k] = -inf;
+    }
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+        const int e = tid + p * NT;
+        const uint64_t g = e < S ? i0 + e : j0 + (e - S);
+        live[p] = g < n;
+        finite[p] = live[p];
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) v[p][k] = live[p] ? c[g * DIM + k] : 0.0f;
+        v[p][DIM] = live[p] ? rad[g] : 0.0f;
+#pragma unroll
+        for (int k = 0; k <= DIM; ++k) finite[p] = finite[p] && fabsf(v[p][k]) < inf;
+        if (finite[p]) {
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) {
+                lo[k] = fminf(lo[k], v[p][k]);
+                hi[k] = fmaxf(hi[k], v[p][k]);
+            }
+            rmax = fmaxf(rmax, fabsf(v[p][DIM]));
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        const float a = redux_min(lo[k]), b = redux_max(hi[k]);
+        if (lane == 0) {
+            s_red[warp][2 * k] = a;
+            s_red[warp][2 * k + 1] = b;
+        }
+    }
+    rmax = redux_max(rmax);
+    if (lane == 0) s_red[warp][2 * DIM] = rmax;
+    bool odd = false;  // an infinite or NaN value
+#pragma unroll
+    for (int p = 0; p < PER; ++p) odd = odd || (live[p] && !finite[p]);
+    odd = __syncthreads_or(odd);
+    float c0[DIM], extent = 0.0f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) extent = fmaxf(extent, s_red[w][2 * DIM]);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        float a = inf, b = -inf;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            a = fminf(a, s_red[w][2 * k]);
+            b = fmaxf(b, s_red[w][2 * k + 1]);
+        }
+        c0[k] = a <= b ? 0.5f * a + 0.5f * b : 0.0f;
+        if (a <= b) extent = fmaxf(extent, fmaxf(b - c0[k], c0[k] - a));
+    }
+    // sigma extent in [8, 16)
+    const bool usable = extent >= 8.8817842e-16f && extent <= 1.1529215e18f;  // [2^-50, 2^60]
+    const float sigma = usable ? __uint_as_float((uint32_t)(257 - (int)(__float_as_uint(extent) >> 23)) << 23) : 0.0f;
+#pragma unroll
+    for (int p = 0; p < PER; ++p) {
+        const int e = tid + p * NT;
+        const bool ok = finite[p] && usable, column = S >= NT ? p >= S / NT : e >= S;
+        // sigma c - sigma c0 rounds once, as sigma (c - c0) does: sigma is a power of two
+        float X[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) X[k] = 0.0f;
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) X[k] = ok ? fmaf(v[p][k], sigma, -sigma * c0[k]) : 0.0f;
+        X[3] = ok ? v[p][DIM] * sigma : 0.0f;
+        float u = X[3] * X[3];
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) u = fmaf(-X[k], X[k], u);
+        u = ok ? fmaf(0.5f, u, 0.001953125f) : (live[p] ? 30000.0f : -30000.0f);
+        const uint32_t h0 = half2_bits(X[0], X[1]), h1 = half2_bits(X[2], X[3]);
+        const float2 f0 = half2_floats(h0), f1 = half2_floats(h1);
+        const uint32_t l0 = half2_bits(X[0] - f0.x, X[1] - f0.y), l1 = half2_bits(X[2] - f1.x, X[3] - f1.y);
+        const float uh = __half2float(__float2half_rn(u));
+        const uint32_t uu = half2_bits(uh, u - uh), one = 0x3C003C00u;
+        // rows (hi, hi, lo, u, 1) against columns (hi, lo, hi, 1, u)
+        rec[2 * e] = column ? make_uint4(h0, h1, l0, l1) : make_uint4(h0, h1, h0, h1);
+        rec[2 * e + 1] = column ? make_uint4(h0, h1, one, uu) : make_uint4(l0, l1, uu, one);
+        pos[e] = make_float4(v[p][0], DIM > 1 ? v[p][DIM > 1 ? 1 : 0] : 0.0f, DIM > 2 ? v[p][DIM > 2 ? 2 : 0] : 0.0f, v[p][DIM]);
+    }
+    __syncthreads();
+
+    // A thread of quad t = lane % 4 takes words 2t and 2t + 1 of a record: the
+    // inner index is permuted alike in both operands.
+    const uint2 *words = reinterpret_cast<const uint2 *>(rec);
+    constexpr int RG = S / 64, CS = NW / RG;             // row groups, warps per row group
+    const int r0 = (warp % RG) * 64, part = warp / RG;   // this warp's rows, its share of the columns
+    const int g = lane >> 2, t = lane & 3;
+    uint2 a[4][2];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        a[m][0] = words[(r0 + 16 * m + g) * 4 + t];
+        a[m][1] = words[(r0 + 16 * m + 8 + g) * 4 + t];
+    }
+    // a diagonal block needs no column past the group's last row
+    const int jn = bi == bj ? (r0 + 64) / 8 : S / 8;
+    const uint2 *bw = words + S * 4;
+    uint32_t d[4][4];
+    auto filter = [&](int jt) {
+        const uint2 b = bw[(jt * 8 + g) * 4 + t];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) mma_16x8x16(a[m][0], a[m][1], b, d[m]);
+        uint32_t acc = d[0][0];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc &= d[m][0] & d[m][1] & d[m][2] & d[m][3];
+        return (int)acc >= 0;
+    };
+    // bit 4 m + e: the value of row 16 m + g + 8 (e / 2), column 2 t + (e & 1) is not negative
+    auto flags = [&]() {
+        uint32_t mask = 0;
+#pragma unroll
+        for (int m = 0; m < 4; ++m)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) mask |= (~d[m][e] >> 31) << (4 * m + e);
+        return mask;
+    };
+    // the trial: flags among each warp's first 512 pairs
+    uint32_t first = part < jn && filter(part) ? __popc(flags()) : 0u;
+    first = __reduce_add_sync(FULL, first);
+    if (lane == 0) s_flags[warp] = first;
+    __syncthreads();
+    uint32_t total = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) total += s_flags[w];
+    if (total > NW * 512 / 128 && usable && !odd) {
+        constexpr int Q = S / 128;  // packed FP32 tiles a side
+        for (int w = 0; w < Q * Q; ++w) {
+            const uint32_t ti = bi * Q + w / Q, tj = bj * Q + w % Q;
+            if (tj > ti || (uint64_t)ti * 128 >= n) continue;
+            __syncthreads();  // the previous tile's spheres have been read
+            collide_tile<16, 8, DIM>(c, rad, n, ti, tj, o, tid & 15, tid >> 4);
+        }
+        return;
+    }
+    uint32_t hits = 0;
+    for (int jt = part; jt < jn; jt += CS) {
+        if (!__any_sync(FULL, filter(jt))) continue;
+        for (uint32_t mask = flags(); mask; mask &= mask - 1) {
+            const int bit = __ffs(mask) - 1;
+            const int r = r0 + 16 * (bit >> 2) + g + 8 * ((bit >> 1) & 1), q = jt * 8 + 2 * t + (bit & 1);
+            const uint64_t i = i0 + r, j = j0 + q;
+            if (i >= n || j >= i) continue;
+            const float4 pi = pos[r], pj = pos[S + q];
+            const float va[4] = {pi.x, pi.y, pi.z, pi.w}, vb[4] = {pj.x, pj.y, pj.z, pj.w};
+            float fa[DIM + 1], fb[DIM + 1];
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) {
+                fa[k] = va[k];
+                fb[k] = vb[k];
+            }
+            fa[DIM] = va[3];
+            fb[DIM] = vb[3];
+            if (!hit_scalar<DIM>(fa, fb)) continue;
+            if (o.pairs) {
+                record(o, (uint32_t)i, (uint32_t)j);
+            } else {
+                ++hits;
+                if (o.count) {
+                    atomicAdd(o.count + i, 1u);
+                    atomicAdd(o.count + j, 1u);
+                }
+            }
+        }
+    }
+    // without a list the pairs are only counted: one atomic per warp, not one per pair
+    const uint32_t w = __reduce_add_sync(FULL, hits);
+    if (lane == 0 && w) atomicAdd(o.n_pairs, (unsigned long long)w);
+}
+
+template <int MAP, int S, int DIM>
+__global__ void __launch_bounds__(MMA_THREADS, MMA_BLOCKS)
+    collide_mma_kernel(const float *__restrict__ c, const float *__restrict__ rad, uint32_t n, CollideOut o,
+                       BlockMap bm)
+{
+    uint32_t bi, bj;
+    if (!map_block<MAP>(bm, bi, bj)) return;
+    collide_tile_mma<S, DIM>(c, rad, n, bi, bj, o);
+}
+
+// Zeroes the outputs in one launch (two memsets cost two).
+__global__ void collide_zero_kernel(uint32_t *__restrict__ count, uint32_t n, unsigned long long *__restrict__ n_pairs)
+{
+    const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t == 0) *n_pairs = 0ull;
+    if (count && t < n) count[t] = 0u;
+}
+
+template <int S, int DIM>
+int launch_mma(const float *c, const float *rad, uint32_t n, int map, CollideOut o, cudaStream_t s)
+{
+    const uint32_t m = (uint32_t)(((uint64_t)n + S - 1) / S);
+    constexpr int smem = 2 * S * 48;
+    return trihost::map_launches(map, m, [&](auto tag, dim3 g, const BlockMap &bm) -> cudaError_t {
+        constexpr int MAP = decltype(tag)::value;
+        if constexpr (MAP != MAP_REC) {
+            if (smem > 40 * 1024) {
+                const cudaError_t e = cudaFuncSetAttribute(collide_mma_kernel<MAP, S, DIM>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                if (e != cudaSuccess) return e;
+            }
+            collide_mma_kernel<MAP, S, DIM><<<g, MMA_THREADS, smem, s>>>(c, rad, n, o, bm);
+            return cudaGetLastError();
+        }
+        return cudaErrorInvalidValue;
+    });
+}
+
+// Tile side: the staging of 2 S spheres pays off over S^2 pairs, so the largest
+// tile that still gives every SM several blocks.
+template <int DIM>
+int launch_filter(const float *c, const float *rad, uint32_t n, int map, CollideOut o, cudaStream_t s)
+{
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const auto blocks = [&](uint64_t S) { return T2((n + S - 1) / S); };
+    if (blocks(512) >= 4ull * nsm) return launch_mma<512, DIM>(c, rad, n, map, o, s);
+    if (blocks(256) >= 2ull * nsm) return launch_mma<256, DIM>(c, rad, n, map, o, s);
+    return launch_mma<128, DIM>(c, rad, n, map, o, s);
+}
+
 // 8 x 8 pairs per thread on 16 x 16 threads: registers capped at 64 so that
 // four blocks share an SM (uncapped the tile takes over 100 and three fit,
 // which leaves too few warps to cover the staging loads).
@@ -166,7 +482,7 @@ __global__ void __launch_bounds__(RHO *RHO, (RHO == 16 && R == 8) ? 4 : 1)
 {
     uint32_t bi, bj;
     if (!map_block<MAP>(bm, bi, bj)) return;
-    collide_tile<RHO, R, DIM>(c, rad, n, bi, bj, o);
+    collide_tile<RHO, R, DIM>(c, rad, n, bi, bj, o, threadIdx.x, threadIdx.y);
 }
 
 // UTM (Section 4.2): thread k of the (n+1) n / 2 pairs j <= i, one test each,
@@ -228,6 +544,11 @@ extern "C" int tri_collide(const float *centres, const float *radii, uint32_t n,
 {
     if ((n && (!centres || !radii)) || !n_pairs || (!pairs && pair_cap > 0)) return TRI_EINVAL;
     if (dim < 1 || dim > 3 || !trihost::rho_ok(rho)) return TRI_EINVAL;
+    // reg = 0, the library's choice: the tensor-core filter for 2-D and 3-D spheres
+    // and the maps that place any number of block rows.  Its tiles are larger, so a size it covers
+    // is first checked against the packed tile's block rows, which the other
+    // maps run at.
+    const bool filter = reg == 0 && dim >= 2 && map != TRI_MAP_REC && map != TRI_MAP_UTM;
     if (reg == 0) reg = rho <= 16 ? 8 : 4;
     if ((reg != 1 && reg != 4 && reg != 8) || (reg == 8 && rho > 16)) return TRI_EINVAL;
     if (map < TRI_MAP_LAMBDA || map > TRI_MAP_LAMBDA_PDELTA) return TRI_EINVAL;
@@ -238,10 +559,16 @@ extern "C" int tri_collide(const float *centres, const float *radii, uint32_t n,
         if (st != TRI_OK) return st;
     }
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(n_pairs, 0, sizeof(*n_pairs), s) != cudaSuccess) return TRI_ECUDA;
-    if (count && n && cudaMemsetAsync(count, 0, sizeof(uint32_t) * n, s) != cudaSuccess) return TRI_ECUDA;
+    collide_zero_kernel<<<(unsigned)((count ? (uint64_t)n : 0) / 256 + 1), 256, 0, s>>>(count, n, n_pairs);
+    if (cudaGetLastError() != cudaSuccess) return TRI_ECUDA;
     if (n == 0) return TRI_OK;
     const CollideOut o{count, pairs, pairs ? pair_cap : 0, n_pairs};
+    if (filter) {
+        switch (dim) {
+        case 2: return launch_filter<2>(centres, radii, n, map, o, s);
+        default: return launch_filter<3>(centres, radii, n, map, o, s);
+        }
+    }
     switch (dim) {
     case 1: return launch_dim<1>(centres, radii, n, map, rho, reg, o, s);
     case 2: return launch_dim<2>(centres, radii, n, map, rho, reg, o, s);

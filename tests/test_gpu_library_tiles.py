@@ -11,6 +11,70 @@ from paper_1609_01490_gb300 import inputs
 pytestmark = pytest.mark.gpu
 
 
+# --------------------------------------------------------------- collisions --
+def _collide(c, r, map_id, cap):
+    import torch
+    t, D, n = tri(), dev(), c.shape[0]
+    npairs = torch.full((1,), 9, dtype=torch.int64, device=D)
+    count = torch.full((n,), 7, dtype=torch.int32, device=D)
+    pairs = torch.zeros((cap, 2), dtype=torch.int32, device=D) if cap else None
+    t.tri_collide(torch.from_numpy(np.ascontiguousarray(c)).to(D), torch.from_numpy(np.ascontiguousarray(r)).to(D),
+                  npairs, count=count, pairs=pairs, map=map_id)
+    torch.cuda.synchronize()
+    pl = pairs[:int(npairs.item())].cpu().numpy().astype(np.int64) if cap else None
+    return int(npairs.item()), count.cpu().numpy().astype(np.uint32), pl
+
+
+def _check_collide(orc, c, r, maps=("LAMBDA",)):
+    cnt_ref, pi, pj = orc.collide_counts(c, r)
+    n = c.shape[0]
+    for name in maps:
+        for cap in (0, len(pi) + 1):
+            tot, cnt, pl = _collide(c, r, getattr(tri(), "MAP_" + name), cap)
+            assert tot == len(pi), (name, cap)
+            np.testing.assert_array_equal(cnt, cnt_ref)
+            if cap:
+                np.testing.assert_array_equal(np.sort(pl[:, 0] * n + pl[:, 1]), np.sort(pi * n + pj))
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 127, 128, 129, 257, 1000])
+def test_collide_filter_tile_edges(orc, dim, n):
+    c, r = inputs.spheres(n, dim, kappa=8.0, seed=n + dim)
+    _check_collide(orc, c, r, ("LAMBDA", "LAMBDA_PDELTA", "BB", "RB", "REC") if n <= 128 else ("LAMBDA", "BB"))
+
+
+@pytest.mark.parametrize("n", [6400, 18000])  # 256- and 512-sphere tiles
+def test_collide_filter_larger_tiles(orc, n):
+    c, r = inputs.spheres(n, 3, kappa=4.0, seed=n)
+    _check_collide(orc, c, r, ("LAMBDA", "RB"))
+
+
+@pytest.mark.parametrize("case", ["offset", "tiny", "huge", "overflow", "crowd", "special", "point"])
+def test_collide_filter_scales(orc, case):
+    # far from the origin, extents at and past the filter's range, most spheres in a
+    # small part of the extent (which gives the filter up), infinities and NaNs
+    c, r = inputs.spheres(700, 3, kappa=10.0, seed=11)
+    if case == "offset":
+        c = (c + np.float32(3000.0)).astype(np.float32)
+    elif case == "tiny":
+        c, r = (c * np.float32(2.0 ** -70)).astype(np.float32), (r * np.float32(2.0 ** -70)).astype(np.float32)
+    elif case == "huge":
+        c, r = (c * np.float32(2.0 ** 59)).astype(np.float32), (r * np.float32(2.0 ** 59)).astype(np.float32)
+    elif case == "overflow":
+        c, r = (c * np.float32(2.0 ** 100)).astype(np.float32), (r * np.float32(2.0 ** 100)).astype(np.float32)
+    elif case == "crowd":
+        c = c.copy()
+        c[::97] *= np.float32(4000.0)
+    elif case == "special":
+        c, r = c.copy(), r.copy()
+        c[5, 1], c[140, 0], r[33], r[300] = np.inf, np.nan, np.inf, np.nan
+    else:
+        c = np.full_like(c, 0.25)
+    with np.errstate(all="ignore"):
+        _check_collide(orc, c, r)
+
+
 # ------------------------------------------------------------ FP32 distances --
 @pytest.mark.parametrize("prec", ["BF16X6", "BF16X3"])
 def test_tc_edm_row_scales(orc, prec):
