@@ -93,3 +93,45 @@ def test_tc_edm_row_scales(orc, prec):
     ws = torch.empty(t.tri_edm_workspace_size(n, d, p), dtype=torch.uint8, device=D)
     t.tri_edm(torch.from_numpy(x).to(D), out, prec=p, workspace=ws)
     assert rel_err(out.cpu().numpy(), orc.edm_packed(x)) <= 1e-5
+
+
+# --------------------------------------------------------------------- Life --
+@pytest.mark.parametrize("mapname", ["LAMBDA", "LAMBDA_PDELTA", "BB", "RB", "REC"])
+@pytest.mark.parametrize("n", [60, 95, 112, 113, 192, 224, 240, 337, 448, 1000])
+def test_life_long_runs_at_tile_edges(orc, mapname, n):
+    # 96- and 112-cell tiles: sizes around them, more than 16 steps, cells of any
+    # non-zero byte, junk outside the domain that must come back unchanged
+    import torch
+    t, D = tri(), dev()
+    m = -(-n // 128)
+    if mapname == "REC" and m & (m - 1):
+        pytest.skip("REC needs a power of two of 128-cell block rows")
+    ld = -(-n // 16) * 16 + 16
+    g = inputs.ca_grid(n, seed=n, ld=ld)
+    g[g != 0] = np.arange(1, 256, dtype=np.uint8)[np.arange(int((g != 0).sum())) % 255]
+    g[np.triu_indices(n, 1)] = 5
+    g[:, n:] = 9
+    a = torch.from_numpy(g).to(D)
+    for steps in (17, 24, 33, 50):
+        out, scratch = a.clone(), torch.full_like(a, 7)
+        t.tri_ca_run(a, out, n, steps, scratch=scratch, map=getattr(t, "MAP_" + mapname))
+        assert np.array_equal(out.cpu().numpy(), orc.ca_run(g, steps)), steps
+        s = scratch.cpu().numpy()
+        assert np.all(s[np.triu_indices(n, 1)] == 7) and np.all(s[:, n:] == 7)
+
+
+@pytest.mark.parametrize("n", [5999, 6001, 9000])
+def test_life_long_runs_match_single_steps(n):
+    # both halos at sizes with many tiles, against step-by-step tri_ca_step
+    import torch
+    t, D = tri(), dev()
+    ld = -(-n // 16) * 16
+    a = torch.randint(0, 2, (n, ld), generator=torch.Generator(device=D).manual_seed(n), device=D, dtype=torch.uint8).tril_()
+    out, scratch, p, q = (torch.zeros_like(a) for _ in range(4))
+    t.tri_ca_run(a, out, n, 35, scratch=scratch)
+    src = a
+    for s in range(35):
+        dst = q if s & 1 else p
+        t.tri_ca_step(src, dst, n, rho=32)
+        src = dst
+    assert torch.equal(out, src)
