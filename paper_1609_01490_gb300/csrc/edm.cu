@@ -3,6 +3,7 @@
 // in edm_tile.cuh; many uneven triangles in one launch are in edm_batched.cu.
 #include <cuda_runtime.h>
 
+#include "edm_rows.cuh"
 #include "edm_tile.cuh"
 #include "tri_internal.h"
 
@@ -18,6 +19,31 @@ __global__ void __launch_bounds__(RHO *RHO) edm_kernel(const float *__restrict__
     uint32_t bi, bj;
     if (!map_block<MAP>(bm, bi, bj)) return;
     edm_tile<RHO, R, PIPE>(x, n, d, out, bi, bj);
+}
+
+template <int MAP, int D>
+__global__ void __launch_bounds__(rows::THREADS) edm_rows_kernel(const float *__restrict__ x, uint32_t n, uint32_t d,
+                                                                 float *__restrict__ out, BlockMap bm)
+{
+    uint32_t bi, bj;
+    if (!map_block<MAP>(bm, bi, bj)) return;
+    rows::tile<D>(x, n, d, out, bi, bj);
+}
+
+int launch_rows(const float *x, uint32_t n, uint32_t d, float *out, int map, cudaStream_t s)
+{
+    const uint32_t m = (uint32_t)(((uint64_t)n + rows::S - 1) / rows::S);
+    return trihost::map_launches(map, m, [&](auto tag, dim3 g, const BlockMap &bm) -> cudaError_t {
+        constexpr int MAP = decltype(tag)::value;
+        if constexpr (MAP != MAP_REC) {
+            if (d <= 2) edm_rows_kernel<MAP, 2><<<g, rows::THREADS, 0, s>>>(x, n, d, out, bm);
+            else if (d == 3) edm_rows_kernel<MAP, 3><<<g, rows::THREADS, 0, s>>>(x, n, d, out, bm);
+            else if (d == 4) edm_rows_kernel<MAP, 4><<<g, rows::THREADS, 0, s>>>(x, n, d, out, bm);
+            else edm_rows_kernel<MAP, 8><<<g, rows::THREADS, 0, s>>>(x, n, d, out, bm);
+            return cudaGetLastError();
+        }
+        return cudaErrorInvalidValue;
+    });
 }
 
 // UTM is a thread-space map: one thread per pair, no tile to stage.
@@ -74,7 +100,8 @@ cudaError_t launch_rr(uint32_t rho, uint32_t reg, dim3 g, cudaStream_t s, const 
 int trihost::edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int map, uint32_t rho, uint32_t reg,
                       cudaStream_t s)
 {
-    if (reg == 0) reg = 4;  // 4 x 4 pairs per thread: fastest at every d measured (3, 64, 128)
+    const bool choose = reg == 0;  // the library's choice of the tile
+    if (choose) reg = 4;
     // 8 x 8 pairs per thread only with rho <= 16 (registers and shared memory)
     if ((reg != 1 && reg != 2 && reg != 4 && reg != 8) || (reg == 8 && rho > 16)) return TRI_EINVAL;
     if (map == TRI_MAP_UTM) {
@@ -82,6 +109,23 @@ int trihost::edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int ma
         if (total > 0xFFFFFFFFull) return TRI_ERANGE;
         edm_utm_kernel<<<trihost::linear_grid((total + tpb - 1) / tpb), dim3(rho, rho), 0, s>>>(x, n, d, out);
         return cudaGetLastError() == cudaSuccess ? TRI_OK : TRI_ECUDA;
+    }
+    if (choose && map != TRI_MAP_REC) {
+        // a size that the 4 x 4 tile's block rows put out of the map's range stays
+        // out of it; REC keeps that tile, whose block rows it needs a power of two of
+        const int st = trihost::map_range(map, ((uint64_t)n + 4 * rho - 1) / (4 * rho));
+        if (st != TRI_OK) return st;
+        // few features: the row tile once there are several of its blocks per SM
+        // (d = 3: n = 65536 2350 -> 1718 us, n = 8000 41 -> 33; n = 4000 ties at 14.4,
+        // n = 2048 would go from 8.1 to 10.3)
+        if (d <= (uint32_t)rows::MAX_D && T2(((uint64_t)n + rows::S - 1) / rows::S) >= 800)
+            return launch_rows(x, n, d, out, map, s);
+        // many features (more than one 32-feature pass): 8 x 8 pairs per thread, bound
+        // by arithmetic with half the shared-memory reads per pair, once there are
+        // three blocks per SM (rho = 16, d = 100: n = 20011 2071 -> 1562 us, n = 4000
+        // 94 -> 84; n = 2500 would go from 43 to 45.  d = 32: equal within 2%)
+        const uint64_t m8 = ((uint64_t)n + 8 * rho - 1) / (8 * rho);
+        if (rho <= 16 && d > (uint32_t)KC && T2(m8) >= 500) reg = 8;
     }
     const uint32_t S = rho * reg;
     const uint32_t m = (n + S - 1) / S;

@@ -76,6 +76,39 @@ def test_collide_filter_scales(orc, case):
 
 
 # ------------------------------------------------------------ FP32 distances --
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("n", [1, 3, 125, 126, 127, 128, 129, 256, 383, 700])
+def test_edm_row_tiles(d, n):
+    # the same operations per pair as the 4 x 4 tile: the same bits, at every
+    # alignment of the output, and nothing written around it
+    import torch
+    t, D = tri(), dev()
+    x = torch.from_numpy(inputs.edm_normal_points(n, d, seed=n + d)).to(D)
+    size = n * (n + 1) // 2
+    ref = torch.empty(size, device=D)
+    t.tri_edm(x, ref, reg=4)
+    for name in ("LAMBDA", "LAMBDA_PDELTA", "BB", "RB"):
+        for off in range(4):
+            buf = torch.full((size + 16,), -7.0, device=D)
+            t.tri_edm(x, buf[8 + off:8 + off + size], map=getattr(t, "MAP_" + name))
+            assert torch.equal(buf[8 + off:8 + off + size], ref), (name, off)
+            assert bool((buf[:8 + off] == -7.0).all()) and bool((buf[8 + off + size:] == -7.0).all())
+
+
+@pytest.mark.parametrize("d", [9, 16, 33, 100])
+def test_edm_chosen_square_tiles(d):
+    # sizes on both sides of the choice between 4 x 4 and 8 x 8 pairs per thread
+    import torch
+    t, D = tri(), dev()
+    for n in (300, 5000):
+        x = torch.from_numpy(inputs.edm_normal_points(n, d, seed=n + d)).to(D)
+        a, b = (torch.empty(n * (n + 1) // 2, device=D) for _ in range(2))
+        for rho in (8, 16, 32):
+            t.tri_edm(x, a, rho=rho)
+            t.tri_edm(x, b, rho=rho, reg=4)
+            assert torch.equal(a, b), (n, rho)
+
+
 @pytest.mark.parametrize("prec", ["BF16X6", "BF16X3"])
 def test_tc_edm_row_scales(orc, prec):
     # rows from 2^-40 to 2^40, zero rows, rows whose largest feature dwarfs the
