@@ -168,3 +168,24 @@ def test_life_long_runs_match_single_steps(n):
         t.tri_ca_step(src, dst, n, rho=32)
         src = dst
     assert torch.equal(out, src)
+
+
+# --------------------------------------------------------------- cost model --
+@pytest.mark.parametrize("B,F,H1,H2", [(1, 1, 1, 1), (3, 14, 16, 17), (5, 64, 128, 128), (128, 15, 16, 31), (129, 14, 64, 64),
+                                       (1030, 14, 33, 96)])
+def test_mlp_shapes(orc, B, F, H1, H2):
+    import torch
+    t, D = tri(), dev()
+    rng = np.random.default_rng(B + F)
+    theta = (rng.normal(size=orc.mlp_nparams(F, H1, H2)) * 0.2).astype(np.float32)
+    X, y = rng.normal(size=(B, F)).astype(np.float32), rng.normal(size=B).astype(np.float32)
+    th, Xd, yd = (torch.from_numpy(a).to(D) for a in (theta, X, y))
+    ws = torch.empty(t.tri_mlp_workspace_size(B, H1, H2) // 4, device=D)
+    pred, loss, grad = torch.empty(B, device=D), torch.empty(1, device=D), torch.full_like(th, 9.0)
+    t.tri_mlp_forward(th, Xd, pred, H1, H2, ws)
+    t.tri_mlp_grad(th, Xd, yd, loss, grad, H1, H2, ws)
+    # sums of at most 129 products and of B terms in FP32: 1e-4 of the scale, as for the fixed shape
+    np.testing.assert_allclose(pred.cpu().numpy(), orc.mlp_forward(theta.astype(np.float64), X, H1, H2), rtol=1e-4, atol=1e-5)
+    ref_loss, ref_g = orc.mlp_grad(theta.astype(np.float64), X, y, H1, H2)
+    assert float(loss.item()) == pytest.approx(ref_loss, rel=1e-5)
+    assert np.max(np.abs(grad.cpu().numpy().astype(np.float64) - ref_g)) <= 1e-4 * np.max(np.abs(ref_g))
