@@ -308,6 +308,21 @@ static int ca_args_ok(const uint8_t *in, const uint8_t *out, uint32_t n, size_t 
     return TRI_OK;
 }
 
+// The tile a whole-grid step runs at (the result does not depend on it).  Large
+// grids under Conway's rule take 128 x 128 cells whatever rho: blocks of four
+// warps that prefetch ahead, against one-warp blocks bound by load latency (lambda,
+// rho = 16 / 32: n = 16384 75 / 56 us, 8000 21.6 / 19.0, 6000 12.6 / 12.4, 4096
+// 7.4 / 8.5).  Other rules keep sixteen-cell strips of a whole row per thread
+// group, and at rho = 32 the ten rows a thread holds cost it its occupancy: 64 x
+// 64 cells take 96 us there instead of 140 (n = 4096: 9.8 / 12.7, 900: 4.7 / 8.1).
+// REC is placed over its own block rows and keeps its tile.
+static uint32_t step_rho(uint32_t n, uint32_t table, int map, uint32_t rho)
+{
+    if (map == TRI_MAP_REC) return rho;
+    if (table == LIFE_TABLE) return n >= 6000 ? 32 : rho;
+    return rho == 32 ? 16 : rho;
+}
+
 extern "C" int tri_ca_step(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld, uint32_t birth_mask,
                            uint32_t survive_mask, int map, uint32_t rho, void *stream)
 {
@@ -315,6 +330,7 @@ extern "C" int tri_ca_step(const uint8_t *in, uint8_t *out, uint32_t n, size_t l
     if (ok != TRI_OK) return ok;
     const uint32_t table = birth_mask | (survive_mask << 9);  // bit count + 9*alive
     cudaStream_t s = (cudaStream_t)stream;
+    rho = step_rho(n, table, map, rho);
     const uint32_t S = 4 * rho, m = (n + S - 1) / S;
     BlockMap bm{};
     bm.m = m;

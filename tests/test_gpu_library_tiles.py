@@ -170,6 +170,22 @@ def test_life_long_runs_match_single_steps(n):
     assert torch.equal(out, src)
 
 
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 128, 129, 1000, 3001])
+@pytest.mark.parametrize("rho", [8, 16, 32])
+def test_life_step_default_tiles(orc, n, rho):
+    import torch
+    t, D = tri(), dev()
+    ld = -(-n // 16) * 16
+    g = inputs.ca_grid(n, seed=n, ld=ld)
+    g[np.triu_indices(n, 1)] = 5
+    a = torch.from_numpy(g).to(D)
+    ref = orc.ca_step(g)
+    for name in ("LAMBDA", "BB", "RB"):
+        out = a.clone()
+        t.tri_ca_step(a, out, n, map=getattr(t, "MAP_" + name), rho=rho)
+        assert np.array_equal(out.cpu().numpy(), ref), name
+
+
 # --------------------------------------------------------------- cost model --
 @pytest.mark.parametrize("B,F,H1,H2", [(1, 1, 1, 1), (3, 14, 16, 17), (5, 64, 128, 128), (128, 15, 16, 31), (129, 14, 64, 64),
                                        (1030, 14, 33, 96)])
