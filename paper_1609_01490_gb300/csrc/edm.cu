@@ -116,16 +116,16 @@ int trihost::edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int ma
         const int st = trihost::map_range(map, ((uint64_t)n + 4 * rho - 1) / (4 * rho));
         if (st != TRI_OK) return st;
         // few features: the row tile once there are several of its blocks per SM
-        // (d = 3: n = 65536 2350 -> 1718 us, n = 8000 41 -> 33; n = 4000 ties at 14.4,
-        // n = 2048 would go from 8.1 to 10.3)
+        // (d = 3: n = 65536 1997 us with 4 x 4 pairs a thread, 1718 with it; n = 4000
+        // ties at 14.4, n = 2048 would go from 8.1 to 10.3)
         if (d <= (uint32_t)rows::MAX_D && T2(((uint64_t)n + rows::S - 1) / rows::S) >= 800)
             return launch_rows(x, n, d, out, map, s);
-        // many features (more than one 32-feature pass): 8 x 8 pairs per thread, bound
-        // by arithmetic with half the shared-memory reads per pair, once there are
-        // three blocks per SM (rho = 16, d = 100: n = 20011 2071 -> 1562 us, n = 4000
-        // 94 -> 84; n = 2500 would go from 43 to 45.  d = 32: equal within 2%)
+        // more features: 8 x 8 pairs per thread, bound by arithmetic with half the
+        // shared-memory reads per pair, once there are three blocks per SM (4 x 4 / 8 x
+        // 8 at rho = 16, us: n = 20011 d = 100 1627 / 1318, d = 32 616 / 488, d = 9 293 /
+        // 238; d = 64 n = 4000 49 / 47, n = 2500 24.4 / 26.9)
         const uint64_t m8 = ((uint64_t)n + 8 * rho - 1) / (8 * rho);
-        if (rho <= 16 && d > (uint32_t)KC && T2(m8) >= 500) reg = 8;
+        if (rho <= 16 && d > (uint32_t)rows::MAX_D && T2(m8) >= 500) reg = 8;
     }
     const uint32_t S = rho * reg;
     const uint32_t m = (n + S - 1) / S;

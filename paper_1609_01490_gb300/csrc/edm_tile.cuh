@@ -31,6 +31,17 @@ struct TileSmem {
     static constexpr size_t bytes(bool pipe) { return sizeof(float) * (pipe ? 2 : 1) * PASS; }
 };
 
+// Where column c of a tile is staged: columns c and c + RHO of each 2 RHO are
+// neighbours, so that a thread's 8-byte load holds one column of each half and a
+// store instruction covers RHO consecutive floats of a row (in natural order it
+// covers every other one of 2 RHO: ten part-written sectors a row pair at RHO =
+// 16 instead of six whole ones).
+template <int RHO, int R>
+__host__ __device__ constexpr uint32_t col_place(uint32_t c)
+{
+    return R == 1 ? c : c / (2 * RHO) * (2 * RHO) + 2 * (c % RHO) + c / RHO % 2;
+}
+
 // Asynchronous 4-byte global -> shared copy (zero-filled when !valid, which
 // then reads nothing).
 __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool valid)
@@ -42,13 +53,13 @@ __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool val
 template <int R>
 struct TileAcc {
     static constexpr int RC = R == 1 ? 1 : R / 2;  // column groups per thread
-    // a[u][v]: packed partial sums of row u with columns c(v) and c(v) + 1
+    // a[u][v]: packed partial sums of row u with columns c(v) and c(v) + RHO
     // (R >= 2); for R = 1 the low half holds the single pair
     unsigned long long a[R][RC];
 };
 
 // Which of a thread's (row u, column group v) accumulators a tile computes.
-// Thread (ty, tx) owns rows ty + u RHO and columns 2 tx + 2 RHO v + {0, 1}.
+// Thread (ty, tx) owns rows ty + u RHO and columns tx + 2 RHO v + {0, RHO}.
 //  - Rows u >= UA lie past the instance's last point: a tile of the last row
 //    block computes only UA = ceil(rows left / RHO) row groups, for every
 //    thread alike.
@@ -102,11 +113,33 @@ __device__ __forceinline__ void tile_pass(const float *si, const float *sj, uint
     }
 }
 
-// The square roots of the thread's live pairs with j <= i < n, to the packed rows.
+// The square roots of the thread's live pairs with j <= i < n, to the packed
+// rows.  A tile below the diagonal whose rows all lie in the grid takes every
+// pair and needs no tests (six of an 8 x 8 thread's 16 instructions per pair).
 template <int RHO, int R, int UA, bool DIAG>
 __device__ __forceinline__ void tile_store(const TileAcc<R> &acc, float *__restrict__ out, uint32_t n, uint64_t i0,
                                            uint64_t j0, int tx, int ty)
 {
+    if constexpr (R >= 2 && UA == R && !DIAG) {
+        if (j0 < i0 && i0 + RHO * R <= n) {
+            float *row = out + T2(i0 + ty) + j0 + tx;
+            // T2(i + RHO) - T2(i) = RHO i + RHO (RHO + 1) / 2
+            uint64_t step = RHO * (i0 + ty) + RHO * (RHO + 1) / 2;
+#pragma unroll
+            for (int u = 0; u < R; ++u) {
+#pragma unroll
+                for (int v = 0; v < TileAcc<R>::RC; ++v) {
+                    float lo, hi;
+                    f2_unpack(acc.a[u][v], lo, hi);
+                    row[2 * RHO * v] = sqrtf(lo);
+                    row[2 * RHO * v + RHO] = sqrtf(hi);
+                }
+                row += step;
+                step += RHO * RHO;
+            }
+            return;
+        }
+    }
 #pragma unroll
     for (int u = 0; u < R; ++u) {
         if (!tile_live<R, UA, DIAG>(u, 0)) continue;
@@ -120,11 +153,11 @@ __device__ __forceinline__ void tile_store(const TileAcc<R> &acc, float *__restr
 #pragma unroll
             for (int v = 0; v < TileAcc<R>::RC; ++v) {
                 if (!tile_live<R, UA, DIAG>(u, v)) continue;
-                const uint64_t j = j0 + 2 * tx + 2 * RHO * v;
+                const uint64_t j = j0 + tx + 2 * RHO * v;
                 float lo, hi;
                 f2_unpack(acc.a[u][v], lo, hi);
                 if (j <= i) row[j] = sqrtf(lo);
-                if (j + 1 <= i) row[j + 1] = sqrtf(hi);
+                if (j + RHO <= i) row[j + RHO] = sqrtf(hi);
             }
         }
     }
@@ -134,14 +167,18 @@ __device__ __forceinline__ void tile_store(const TileAcc<R> &acc, float *__restr
 extern __shared__ __align__(16) float tile_smem[];
 
 // One (RHO R) x (RHO R) tile.  Thread (ty, tx) owns rows ty + u RHO and, for
-// R = 1, column tx; for R >= 2, the column pairs 2 tx + 2 RHO v + {0, 1}
-// (v < R / 2), updated two at a time with f32x2 instructions, so that a
-// warp's 16 threads of a row cover 32 consecutive columns.  The features are
+// R = 1, column tx; for R >= 2, the column pairs tx + 2 RHO v + {0, RHO}
+// (v < R / 2), updated two at a time with f32x2 instructions.  The features are
 // taken KC at a time.  PIPE = false (d <= KC: one pass, nothing to overlap)
 // stages with plain loads and stores into one pass buffer; PIPE = true
 // copies the next pass in asynchronously while the current one is computed
 // (two pass buffers) and ends without a block barrier: a caller that runs
-// another tile in the same block synchronises the block first.  UA and DIAG
+// another tile in the same block synchronises the block first.  What bounds it:
+// the FMA pipe, two operations per pair and feature (n = 20011, d = 100, 8 x 8
+// pairs on 16 x 16 threads: 1318 us, 0.8 of that pipe).  The instructions around
+// them count: with staging addresses formed from 64-bit indices for every float
+// and a bounds test for every pair it took 1562 us (N = 65536, d = 3, 4 x 4:
+// 2350 us against 1997 now; the 1000-instance batch 15.9 ms against 14.0).  UA and DIAG
 // select the live accumulators (tile_live); the caller guarantees that rows
 // from i0 + UA RHO on are past n and, for DIAG, that i0 = j0.
 template <int RHO, int R, bool PIPE, int UA = R, bool DIAG = false>
@@ -150,6 +187,7 @@ __device__ __forceinline__ void edm_tile_body(const float *__restrict__ x, uint3
 {
     using L = TileSmem<RHO, R>;
     constexpr int S = L::S;
+    static_assert(RHO * RHO / KC <= RHO, "a staging sweep stays within one half of a column group");
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * RHO + tx;
     const uint64_t i0 = (uint64_t)bi * S, j0 = (uint64_t)bj * S;
     TileAcc<R> acc;
@@ -160,37 +198,47 @@ __device__ __forceinline__ void edm_tile_body(const float *__restrict__ x, uint3
 
     if constexpr (!PIPE) {
         float *si = tile_smem, *sj = si + KC * L::LI;
-        for (uint32_t k0 = 0; k0 < d; k0 += KC) {
-            const uint32_t kc = min((uint32_t)KC, d - k0);
-            // stage x[i0 + r][k0 + k] and x[j0 + r][k0 + k], transposed to [k][r]
-            for (uint32_t t = tid; t < (uint32_t)S * kc; t += RHO * RHO) {
-                const uint32_t r = t / kc, k = t - r * kc;
-                const uint64_t gi = i0 + r, gj = j0 + r;
-                si[k * L::LI + r] = gi < n ? x[gi * d + k0 + k] : 0.0f;
-                sj[k * L::LJ + r] = gj < n ? x[gj * d + k0 + k] : 0.0f;
+        // d <= KC: the points of the rows and of the columns are contiguous; stage
+        // them transposed to [k][r], a thread walking them NT floats at a time
+        constexpr uint32_t NT = RHO * RHO;
+        const float *pi = x + i0 * d, *pj = x + j0 * d;
+        const uint32_t ni = (uint32_t)min((uint64_t)S, n - min((uint64_t)n, i0)) * d, nj = (uint32_t)min((uint64_t)S, n - min((uint64_t)n, j0)) * d;
+        const uint32_t dr = NT / d, dk = NT - dr * d;
+        uint32_t r = tid / d, k = tid - r * d;
+        for (uint32_t t = tid; t < (uint32_t)S * d; t += NT) {
+            si[k * L::LI + r] = t < ni ? pi[t] : 0.0f;
+            sj[k * L::LJ + col_place<RHO, R>(r)] = t < nj ? pj[t] : 0.0f;
+            r += dr;
+            k += dk;
+            if (k >= d) {
+                k -= d;
+                ++r;
             }
-            __syncthreads();
-            tile_pass<RHO, R, UA, DIAG>(si, sj, kc, tx, ty, acc);
-            __syncthreads();
         }
+        __syncthreads();
+        tile_pass<RHO, R, UA, DIAG>(si, sj, d, tx, ty, acc);
+        __syncthreads();
     } else {
         // copy features [k0, k0 + KC) of the block's rows and columns,
         // transposed to [k][r], into pass buffer b (a warp reads 32
         // consecutive features of one point: one 128-byte line)
+        // (NT / KC rows a sweep, so that a thread keeps its feature and walks
+        // down the rows by a fixed stride)
+        constexpr uint32_t STEP = RHO * RHO / KC;
+        const uint32_t k = tid % KC, r0 = tid / KC;
+        const uint32_t ni = (uint32_t)min((uint64_t)S, n - min((uint64_t)n, i0)), nj = (uint32_t)min((uint64_t)S, n - min((uint64_t)n, j0));
         auto stage = [&](int b, uint32_t k0) {
-            float *si = tile_smem + b * L::PASS, *sj = si + KC * L::LI;
-            const uint32_t kc = min((uint32_t)KC, d - k0);
-            auto one = [&](uint32_t r, uint32_t k) {
-                const uint64_t gi = i0 + r, gj = j0 + r;
-                cp_async4(si + k * L::LI + r, gi < n ? x + gi * d + k0 + k : x, gi < n);
-                cp_async4(sj + k * L::LJ + r, gj < n ? x + gj * d + k0 + k : x, gj < n);
-            };
-            if (kc == KC) {
-                for (uint32_t e = tid; e < (uint32_t)S * KC; e += RHO * RHO) one(e / KC, e % KC);
-            } else {
-                for (uint32_t e = tid; e < (uint32_t)S * kc; e += RHO * RHO) {
-                    const uint32_t r = e / kc;
-                    one(r, e - r * kc);
+            if (k < d - k0) {
+                float *si = tile_smem + b * L::PASS + k * L::LI + r0;
+                float *sj = tile_smem + b * L::PASS + KC * L::LI + k * L::LJ + (R == 1 ? r0 : 2 * r0);
+                const float *pi = x + (i0 + r0) * d + k0 + k, *pj = x + (j0 + r0) * d + k0 + k;
+#pragma unroll
+                for (uint32_t r = 0; r < (uint32_t)S; r += STEP) {
+                    cp_async4(si + r, r0 + r < ni ? pi : x, r0 + r < ni);
+                    // col_place(r0 + r) = 2 r0 + col_place(r): r0 < STEP divides r and is at most RHO
+                    cp_async4(sj + col_place<RHO, R>(r), r0 + r < nj ? pj : x, r0 + r < nj);
+                    pi += (size_t)STEP * d;
+                    pj += (size_t)STEP * d;
                 }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
