@@ -116,8 +116,8 @@ int trihost::edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int ma
         const int st = trihost::map_range(map, ((uint64_t)n + 4 * rho - 1) / (4 * rho));
         if (st != TRI_OK) return st;
         // few features: the row tile once there are several of its blocks per SM
-        // (d = 3: n = 65536 1997 us with 4 x 4 pairs a thread, 1718 with it; n = 4000
-        // ties at 14.4, n = 2048 would go from 8.1 to 10.3)
+        // (d = 3, us, 4 x 4 pairs a thread / row tile: n = 65536 1995 / 1209, n = 8000 32.5 /
+        // 24.9, n = 5000 14.4 / 14.1, n = 4000 10.1 / 10.6, n = 2048 4.7 / 7.8)
         if (d <= (uint32_t)rows::MAX_D && T2(((uint64_t)n + rows::S - 1) / rows::S) >= 800)
             return launch_rows(x, n, d, out, map, s);
         // more features: 8 x 8 pairs per thread, bound by arithmetic with half the
