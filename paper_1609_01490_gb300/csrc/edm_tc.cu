@@ -486,13 +486,6 @@ __device__ __forceinline__ float sqrt_approx(float x)
     return y;
 }
 
-// Three-input minimum (a NaN is ignored, as by fminf).
-__device__ __forceinline__ float min3(float a, float b, float c)
-{
-    float y;
-    asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
-    return y;
-}
 
 // Shared-memory matrix descriptor of a K-major operand with 128-byte swizzle:
 // start address (bits 0-13) and leading byte offset (bits 16-29, unused for

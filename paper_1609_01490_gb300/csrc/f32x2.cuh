@@ -35,4 +35,20 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
     return r;
 }
 
+// Three-input minimum (a NaN is ignored, as by fminf).
+__device__ __forceinline__ float min3(float a, float b, float c)
+{
+    float y;
+    asm("min.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+    return y;
+}
+
+// 1 / sqrt(x) by the MUFU unit, subnormal inputs taken as zero.
+__device__ __forceinline__ float rsqrt_ftz(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 }  // namespace tri

@@ -205,3 +205,24 @@ def test_mlp_shapes(orc, B, F, H1, H2):
     ref_loss, ref_g = orc.mlp_grad(theta.astype(np.float64), X, y, H1, H2)
     assert float(loss.item()) == pytest.approx(ref_loss, rel=1e-5)
     assert np.max(np.abs(grad.cpu().numpy().astype(np.float64) - ref_g)) <= 1e-4 * np.max(np.abs(ref_g))
+
+
+# --------------------------------------------------------------- AT energy --
+@pytest.mark.parametrize("scale,finite", [(1.0, True), (3e-4, True), (1e-7, False)])
+def test_at_small_products(scale, finite):
+    """A regular tetrahedron: its four triplets are alike, and the last point pairs
+    sum over two k at once.  At 1e-7 the products a b c are subnormal and a term
+    exceeds FP32's range, so the energy is infinite."""
+    x = np.array([[1, 1, 1], [1, -1, -1], [-1, 1, -1], [-1, -1, 1]], np.float64) * scale
+    import torch
+    t, D = tri(), dev()
+    p = torch.from_numpy(x.astype(np.float32)).to(D)
+    energy = torch.empty(1, dtype=torch.float64, device=D)
+    ws = torch.empty(t.tet_at_workspace_size(4, 16), dtype=torch.uint8, device=D)
+    t.tet_at_energy(p, energy, rho=16, workspace=ws)
+    if finite:
+        # equilateral side r: (1 + 3/8) / r^9 each; FP32 terms, about 20 roundings
+        want = 4 * 1.375 / (np.sqrt(8.0) * np.float64(np.float32(scale))) ** 9
+        assert abs(energy.item() - want) <= 2e-5 * want
+    else:
+        assert energy.item() == float("inf")
