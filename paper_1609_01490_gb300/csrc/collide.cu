@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "f32x2.cuh"
+#include "pdl.cuh"
 #include "tri_maps.cuh"
 
 using namespace tri;
@@ -180,7 +181,7 @@ __device__ __noinline__ void collide_tile(const float *__restrict__ c, const flo
 // 512 pairs per warp is 4 instructions on the tensor core, 8 three-input ANDs
 // and a vote, against about 50 packed FP32 instructions.
 // 65,536 spheres in 3-D take 218 us against 970 with the packed FP32 tile,
-// 9001 in 2-D 21 against 48.  The tensor core bounds it (one m16n8k16 per SM
+// 9001 in 2-D 18.6 against 48.  The tensor core bounds it (one m16n8k16 per SM
 // takes 1.04 ns: 115 us), then the staging of each block's spheres.
 // The margin is 3e-5 of the block's squared extent, so it flags few pairs unless
 // most spheres crowd into a small part of that extent (or meet many others):
@@ -385,6 +386,7 @@ __device__ __noinline__ void collide_tile_mma(const float *__restrict__ c, const
     uint32_t total = 0;
 #pragma unroll
     for (int w = 0; w < NW; ++w) total += s_flags[w];
+    wait_for_previous();  // the outputs are zeroed from here on
     if (total > NW * 512 / 128 && usable && !odd) {
         constexpr int Q = S / 128;  // packed FP32 tiles a side
         for (int w = 0; w < Q * Q; ++w) {
@@ -443,6 +445,7 @@ __global__ void __launch_bounds__(MMA_THREADS, MMA_BLOCKS)
 // Zeroes the outputs in one launch (two memsets cost two).
 __global__ void collide_zero_kernel(uint32_t *__restrict__ count, uint32_t n, unsigned long long *__restrict__ n_pairs)
 {
+    dependents_may_start();
     const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) *n_pairs = 0ull;
     if (count && t < n) count[t] = 0u;
@@ -461,8 +464,7 @@ int launch_mma(const float *c, const float *rad, uint32_t n, int map, CollideOut
                                                            cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
                 if (e != cudaSuccess) return e;
             }
-            collide_mma_kernel<MAP, S, DIM><<<g, MMA_THREADS, smem, s>>>(c, rad, n, o, bm);
-            return cudaGetLastError();
+            return trihost::launch_behind(collide_mma_kernel<MAP, S, DIM>, g, MMA_THREADS, smem, s, c, rad, n, o, bm);
         }
         return cudaErrorInvalidValue;
     });

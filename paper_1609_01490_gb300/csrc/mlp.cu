@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/tri.h"
+#include "pdl.cuh"
 
 namespace {
 
@@ -34,7 +35,7 @@ __host__ __device__ inline uint32_t pass_floats(uint32_t F, uint32_t H1, uint32_
 // in one launch: a block keeps the weights in shared memory and takes the samples
 // four at a time through all the layers.  The passes are bound by latency (the
 // whole batch of the selector's sweep is 2 Mflop): as ten dependent launches a
-// training step took 113 us at B = 391, H1 = H2 = 64, as three it takes 20.  Each sum runs over
+// training step took 113 us at B = 391, H1 = H2 = 64, as three it takes 19.  Each sum runs over
 // its inputs in increasing order.
 template <bool BACK>
 __global__ void __launch_bounds__(MLP_THREADS)
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(MLP_THREADS)
                     uint32_t H1, uint32_t H2, float *__restrict__ pred, const Batch w)
 {
     extern __shared__ float sm[];
+    tri::dependents_may_start();
     float *W1 = sm, *b1 = W1 + H1 * (F + 1), *W2 = b1 + H1, *b2 = W2 + H2 * (H1 + 1), *W3 = b2 + H2, *b3 = W3 + H2;
     float *x = b3 + 1, *z1 = x + GROUP * F, *z2 = z1 + GROUP * H1, *gz2 = z2 + GROUP * H2, *gout = gz2 + GROUP * H2;
     const uint32_t tid = threadIdx.x;
@@ -128,6 +130,7 @@ __global__ void __launch_bounds__(MLP_THREADS) mlp_wgrad_kernel(const GradArgs g
     const uint32_t tid = threadIdx.x;
     uint32_t tile = blockIdx.x, l = 0;
     while (l < 3 && tile >= ga.layer[l].tiles) tile -= ga.layer[l++].tiles;
+    tri::wait_for_previous();
     if (l == 3) {  // the last block: loss = mean (pred - y)^2
         float *part = &sg[0][0];
         float s = 0.0f;
@@ -317,8 +320,7 @@ extern "C" int tri_mlp_grad(const float *theta, const float *X, const float *y, 
                  {w.g_out, w.z2, gW3, gb3, 1u, H2, 1u, tiles(1u, H2)}},
                 w.pred, y, loss, B};
     const uint32_t blocks = ga.layer[0].tiles + ga.layer[1].tiles + ga.layer[2].tiles + 1;
-    mlp_wgrad_kernel<<<blocks, MLP_THREADS, 0, s>>>(ga);
-    return cudaGetLastError() == cudaSuccess ? TRI_OK : TRI_ECUDA;
+    return trihost::launch_behind(mlp_wgrad_kernel, blocks, MLP_THREADS, 0, s, ga) == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 
 extern "C" int tri_mlp_adam(float *theta, const float *grad, float *m, float *v, uint32_t nparams, uint32_t t,
