@@ -17,7 +17,7 @@
 // 4.8e-8: the planes' rounding costs less than twice the accumulation steps.
 // A pair whose estimate falls below tau (|x_i|^2 + |x_j|^2) has lost
 // too many digits to cancellation and is flagged; a second kernel recomputes
-// flagged pairs in FP64 by direct differences (the paper's definition).
+// flagged pairs by direct differences (the paper's definition).
 //
 // Kernels.  prepare: row norms (FP32 pairs, stored as FP32), row scales and the
 // FP16 planes, K padded to a multiple of 64.  gram: persistent clusters of two CTAs on two
@@ -37,8 +37,11 @@
 // issues its TMA; warps 2-17 of each CTA read TMEM back (lanes = output
 // columns), form the distances, flag cancellations and store the packed rows
 // (one coalesced 128-byte store per warp and row; the four warps that hold the
-// four 32-column quarters of the same rows store them together).  fixup: FP64
-// recompute of the flagged pairs.
+// four 32-column quarters of the same rows store them together).  fixup:
+// recompute of the flagged pairs to FP64's accuracy.  The three kernels of one
+// call are launched behind one another (pdl.cuh) and prepare clears the header,
+// which saves 8 us of a call's five launches (BF16X6, N = 1000, d = 64: 28.6 ->
+// 20.8 us; BF16X3, N = 12345, d = 100 with 1% equal points: 92.7 -> 82.0).
 #include <cuda.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -49,6 +52,7 @@
 #include <mutex>
 
 #include "f32x2.cuh"
+#include "pdl.cuh"
 #include "tri_internal.h"
 #include "tri_maps.cuh"
 
@@ -371,9 +375,12 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 // powers; its inverse goes to scales[].  A row with an infinity or a NaN gets
 // NaN planes there, and NaN distances.
 __global__ void prepare_kernel(const float *__restrict__ x, uint32_t n, uint32_t d, uint32_t dp,
-                               float *__restrict__ norms, float *__restrict__ scales, __half *__restrict__ planes)
+                               float *__restrict__ norms, float *__restrict__ scales, __half *__restrict__ planes,
+                               unsigned long long *__restrict__ header)
 {
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    dependents_may_start();
+    if (warp == 0) header[lane] = 0ull;  // its 256 bytes
     if (warp >= n) return;
     const float *row = x + (size_t)warp * d;
     float hi = 0.0f, lo = 0.0f, big = 0.0f;
@@ -565,6 +572,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
+    dependents_may_start();
+    wait_for_previous();
     tc_fence_before();
     __syncthreads();
     cluster_sync();
@@ -984,18 +993,24 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 }
 
 // -------------------------------------------------------------- fixup ----
-// FP64 direct-difference recompute of the flagged pairs appended since the
-// previous call (list entries [*start, count); all of them when start is
+// Direct-difference recompute of the flagged pairs to FP64's accuracy: sums of
+// squares as FP32 pairs hi + lo (differences exact, about 44 significant bits in
+// the sum), which round to the FP32 distance that an FP64 sum gives; FP64 itself,
+// at a 64th of FP32's rate, only where a sum leaves [2^-60, 2^100] (there squares
+// may vanish or overflow in FP32).  With 123 equal pairs among N =
+// 12345 points FP64 sums, their warps on two SMs, took 20 us; now 2.
+// Takes the list entries appended since the previous call (list entries [*start, count); all of them when start is
 // null).  If the list overflowed, every pair of the packed range [p_begin,
 // p_end) whose stored distance passes a slightly wider version of the flag
 // test is recomputed instead.  next_start (if not null) receives the count,
 // for the next call.
 __global__ void fixup_kernel(const float *__restrict__ x, uint32_t d, float *__restrict__ out,
-                             const float *__restrict__ norms, const unsigned long long *__restrict__ count,
-                             const unsigned long long *__restrict__ list, unsigned long long cap, float tau,
+                             const float *norms, const unsigned long long *count, const unsigned long long *list,
+                             unsigned long long cap, float tau,
                              unsigned long long *n_flagged, const unsigned long long *start,
                              unsigned long long *next_start, uint64_t p_begin, uint64_t p_end)
 {
+    wait_for_previous();
     const unsigned long long cnt = *count, first = start ? *start : 0ull;
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, nth = (uint64_t)gridDim.x * blockDim.x;
     if (tid == 0 && n_flagged) *n_flagged = cnt;
@@ -1019,12 +1034,47 @@ __global__ void fixup_kernel(const float *__restrict__ x, uint32_t d, float *__r
         out[T2(i) + j] = (float)sqrt((s[0] + s[1]) + (s[2] + s[3]));
     };
     if (cnt <= cap) {
-        // one warp per listed pair: lanes take strided features, then a fixed-order tree sum
+        // One warp per listed pair, neighbours in the list on different blocks: lanes
+        // take strided features, then a fixed-order tree sum (the next pair is read
+        // ahead of this one's chain).
         const uint32_t lane = threadIdx.x & 31;
-        for (uint64_t e = first + (tid >> 5); e < cnt; e += nth >> 5) {
-            const unsigned long long v = list[e];
+        uint64_t e = first + (uint64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+        unsigned long long next = e < cnt ? list[e] : 0ull;
+        for (; e < cnt; e += nth >> 5) {
+            const unsigned long long v = next;
+            if (e + (nth >> 5) < cnt) next = list[e + (nth >> 5)];
             const uint32_t i = (uint32_t)(v >> 32), j = (uint32_t)(v & 0xFFFFFFFFu);
             const float *xi = x + (size_t)i * d, *xj = x + (size_t)j * d;
+            float hi = 0.0f, lo = 0.0f;
+            bool apart = false;  // some feature differs (or is NaN)
+            for (uint32_t k = lane; k < d; k += 32) {
+                float f, fe, t, te;
+                two_sum(xi[k], -xj[k], f, fe);
+                apart = apart || !(f == 0.0f);
+                const float p = f * f, pe = fmaf(f + f, fe, fmaf(f, f, -p));  // (f + fe)^2 but for fe^2
+                two_sum(hi, p, t, te);
+                hi = t;
+                lo += te + pe;
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const float oh = __shfl_down_sync(0xffffffffu, hi, o), ol = __shfl_down_sync(0xffffffffu, lo, o);
+                float t, te;
+                two_sum(hi, oh, t, te);
+                hi = t;
+                lo += ol + te;
+            }
+            if (!__any_sync(0xffffffffu, apart)) {
+                if (lane == 0) out[T2(i) + j] = 0.0f;
+                continue;
+            }
+            float sq, sqe;
+            two_sum(hi, lo, sq, sqe);
+            if (__shfl_sync(0xffffffffu, sq >= 8.6736174e-19f && sq <= 1.2676506e30f ? 1 : 0, 0)) {
+                // the root's residual moves the rounded root to that of sq + sqe
+                const float r = sqrtf(sq);
+                if (lane == 0) out[T2(i) + j] = fmaf(fmaf(-r, r, sq) + sqe, 0.5f / r, r);
+                continue;
+            }
             double s = 0.0;
             for (uint32_t k = lane; k < d; k += 32) {
                 const double df = (double)xi[k] - (double)xj[k];
@@ -1094,9 +1144,10 @@ bool plan(uint32_t d, int prec, TcPlan &p)
 
 // Launches the pair kernel on as many CTA pairs as can be resident at once
 // (cached per instantiation and shared-memory size), splitting the units into
-// an up-front run per pair and counter-driven runs.
+// an up-front run per pair and counter-driven runs.  `behind`: right behind
+// tri_edm_prepare's kernel on the same stream.
 template <int MP>
-cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, cudaStream_t s)
+cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, bool behind, cudaStream_t s)
 {
     cudaError_t e = cudaFuncSetAttribute(gram_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -1128,8 +1179,21 @@ cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, cudaSt
     g.static_per = units * STATIC_PCT / 100 / pairs;
     g.dyn_start = g.u0 + g.static_per * pairs;
     g.chunk = DYN_CHUNK;
+    if (behind) return trihost::launch_behind(gram_kernel<MP>, (unsigned)(2 * pairs), NTHREADS, smem, s, tmap, g);
     gram_kernel<MP><<<(unsigned)(2 * pairs), NTHREADS, smem, s>>>(tmap, g);
     return cudaGetLastError();
+}
+
+// The recompute pass, right behind a Gram kernel on the same stream.
+int launch_fixup(const float *x, uint32_t d, float *out, int prec, char *ws, const WsLayout &L,
+                 unsigned long long *n_flagged, const unsigned long long *start, unsigned long long *next_start,
+                 uint64_t p0, uint64_t p1, cudaStream_t s)
+{
+    const cudaError_t e = trihost::launch_behind(
+        fixup_kernel, num_sms() * 4, 256, 0, s, x, d, out, (const float *)(ws + L.norms),
+        (const unsigned long long *)(ws + L.hdr), (const unsigned long long *)(ws + L.flags),
+        (unsigned long long)L.cap, flag_tau(prec, d), n_flagged, start, next_start, p0, p1);
+    return e == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 
 }  // namespace
@@ -1150,19 +1214,19 @@ extern "C" int tri_edm_prepare(const float *x, uint32_t n, uint32_t d, int prec,
     if (!workspace || ws_bytes < L.total || ((uintptr_t)workspace & 255)) return TRI_ENOSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     char *ws = (char *)workspace;
-    if (cudaMemsetAsync(ws, 0, 256, s) != cudaSuccess) return TRI_ECUDA;
     const unsigned blocks = (unsigned)(((uint64_t)n * 32 + 255) / 256);
     prepare_kernel<<<blocks, 256, 0, s>>>(x, n, d, pl.dp, (float *)(ws + L.norms), (float *)(ws + L.scales),
-                                          (__half *)(ws + L.planes));
+                                          (__half *)(ws + L.planes), (unsigned long long *)(ws + L.hdr));
     return cudaGetLastError() == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 
 namespace {
 
 // Unit rows [R0, R1) of the Gram kernel, whose output is the packed rows
-// [256 R0, min(n, 256 R1)).
+// [256 R0, min(n, 256 R1)).  `prepared`: tri_edm_prepare's kernel is the last
+// work on the stream, and has just cleared the unit counter.
 int gram_range(uint32_t n, uint32_t d, float *out, int map, int prec, void *workspace, size_t ws_bytes, uint32_t R0,
-               uint32_t R1, cudaStream_t s)
+               uint32_t R1, bool prepared, cudaStream_t s)
 {
     if (!out || n == 0 || d == 0) return TRI_EINVAL;
     if (n > TC_MAX_N) return TRI_ERANGE;
@@ -1210,9 +1274,9 @@ int gram_range(uint32_t n, uint32_t d, float *out, int map, int prec, void *work
     g.wait_limit = (const unsigned long long *)(ws + L.hdr + 40);
     g.flag_list = (unsigned long long *)(ws + L.flags);
     g.flag_cap = L.cap;
-    if (cudaMemsetAsync(g.tile_counter, 0, sizeof(unsigned long long), s) != cudaSuccess) return TRI_ECUDA;
-    cudaError_t e;
-    e = map == TRI_MAP_LAMBDA ? launch_gram<MAP_LAMBDA>(tmap, g, pl.smem, s) : launch_gram<MAP_BB>(tmap, g, pl.smem, s);
+    if (!prepared && cudaMemsetAsync(g.tile_counter, 0, sizeof(unsigned long long), s) != cudaSuccess) return TRI_ECUDA;
+    const cudaError_t e = map == TRI_MAP_LAMBDA ? launch_gram<MAP_LAMBDA>(tmap, g, pl.smem, prepared, s)
+                                                : launch_gram<MAP_BB>(tmap, g, pl.smem, prepared, s);
     return e == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 
@@ -1223,7 +1287,7 @@ extern "C" int tri_edm_gram(uint32_t n, uint32_t d, float *out, int map, int pre
 {
     if (n == 0) return TRI_EINVAL;
     const uint32_t mb = ((n + TILE - 1) / TILE + 1) / 2;
-    return gram_range(n, d, out, map, prec, workspace, ws_bytes, 0, mb, (cudaStream_t)stream);
+    return gram_range(n, d, out, map, prec, workspace, ws_bytes, 0, mb, false, (cudaStream_t)stream);
 }
 
 extern "C" int tri_edm_fixup(const float *x, uint32_t n, uint32_t d, float *out, int prec, void *workspace,
@@ -1248,9 +1312,10 @@ int trihost::edm_tc(const float *x, uint32_t n, uint32_t d, float *out, int map,
                     size_t ws_bytes, unsigned long long *n_flagged, cudaStream_t s)
 {
     int st = tri_edm_prepare(x, n, d, prec, ws, ws_bytes, s);
-    if (st == TRI_OK) st = tri_edm_gram(n, d, out, map, prec, ws, ws_bytes, s);
-    if (st == TRI_OK) st = tri_edm_fixup(x, n, d, out, prec, ws, ws_bytes, n_flagged, s);
-    return st;
+    if (st == TRI_OK) st = gram_range(n, d, out, map, prec, ws, ws_bytes, 0, ((n + TILE - 1) / TILE + 1) / 2, true, s);
+    if (st != TRI_OK) return st;
+    const WsLayout L = ws_layout(n, d, prec);
+    return launch_fixup(x, d, out, prec, (char *)ws, L, n_flagged, nullptr, nullptr, 0, T2(n), s);
 }
 
 // ------------------------------------------------------ split over ranks ----
@@ -1313,14 +1378,9 @@ extern "C" int tri_edm_rows(const float *x, uint32_t n, uint32_t d, uint32_t row
     const uint64_t p0 = T2(row_begin), p1 = T2(row_end);
     float *base = reinterpret_cast<float *>(reinterpret_cast<uintptr_t>(out_band) - p0 * sizeof(float));
     if ((r = gram_range(n, d, base, map, prec, workspace, ws_bytes, row_begin / unit,
-                        (row_end + unit - 1) / unit, s)) != TRI_OK)
+                        (row_end + unit - 1) / unit, true, s)) != TRI_OK)
         return r;
-    char *ws = (char *)workspace;
-    fixup_kernel<<<num_sms() * 4, 256, 0, s>>>(x, d, base, (const float *)(ws + L.norms),
-                                               (const unsigned long long *)(ws + L.hdr),
-                                               (const unsigned long long *)(ws + L.flags), L.cap, flag_tau(prec, d),
-                                               n_flagged, nullptr, nullptr, p0, p1);
-    return cudaGetLastError() == cudaSuccess ? TRI_OK : TRI_ECUDA;
+    return launch_fixup(x, d, base, prec, (char *)workspace, L, n_flagged, nullptr, nullptr, p0, p1, s);
 }
 
 // ---------------------------------------------------------------- host ----
@@ -1373,17 +1433,11 @@ extern "C" int tri_edm_host(const float *x_host, uint32_t n, uint32_t d, float *
         uint32_t R1 = b + 1 == bands ? mb : (uint32_t)std::ceil(mb * std::sqrt((double)(b + 1) / bands));
         R1 = std::min(std::max(R1, R0 + 1), mb);
         if (R0 >= mb) break;
-        if ((r = gram_range(n, d, out_dev, map, prec, workspace, ws_bytes, R0, R1, s)) != TRI_OK) break;
+        if ((r = gram_range(n, d, out_dev, map, prec, workspace, ws_bytes, R0, R1, b == 0, s)) != TRI_OK) break;
         const uint64_t p0 = T2(std::min<uint64_t>(n, 2ull * TILE * R0)), p1 = T2(std::min<uint64_t>(n, 2ull * TILE * R1));
-        fixup_kernel<<<num_sms() * 4, 256, 0, s>>>(x_dev, d, out_dev, (const float *)(ws + L.norms),
-                                                   (const unsigned long long *)(ws + L.hdr),
-                                                   (const unsigned long long *)(ws + L.flags), L.cap,
-                                                   flag_tau(prec, d), n_flagged, slot + (b & 1),
-                                                   slot + ((b + 1) & 1), p0, p1);
-        if (cudaGetLastError() != cudaSuccess) {
-            r = TRI_ECUDA;
+        if ((r = launch_fixup(x_dev, d, out_dev, prec, ws, L, n_flagged, slot + (b & 1), slot + ((b + 1) & 1), p0, p1,
+                              s)) != TRI_OK)
             break;
-        }
         // the band's rows are final: copy them while the next band computes
         cudaEvent_t ev;
         if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {

@@ -207,6 +207,31 @@ def test_mlp_shapes(orc, B, F, H1, H2):
     assert np.max(np.abs(grad.cpu().numpy().astype(np.float64) - ref_g)) <= 1e-4 * np.max(np.abs(ref_g))
 
 
+@pytest.mark.parametrize("e", [-45, -27, 0, 56])  # sums of squares below 2^-60, about it, ordinary, above 2^100
+@pytest.mark.parametrize("d", [1, 3, 32, 33, 100])
+def test_tc_edm_recomputed_pairs(d, e):
+    """Close and equal pairs are recomputed to within the final rounding (half an
+    ulp; the sum's own error is below 2^-40) at every scale."""
+    import torch
+    t, D = tri(), dev()
+    n, rng = 300, np.random.default_rng(d)
+    a = rng.normal(size=(n // 2, d)) + np.where(rng.random((n // 2, d)) < 0.5, -3.0, 3.0)
+    x = np.stack([a, a + 0.1 * rng.normal(size=a.shape)], 1).reshape(n, d).astype(np.float32)
+    x[1:60:2] = x[0:60:2]
+    x = np.ldexp(x, e).astype(np.float32)
+    xd = torch.from_numpy(x).to(D)
+    out = torch.empty(n * (n + 1) // 2, device=D)
+    flagged = torch.zeros(1, dtype=torch.int64, device=D)
+    ws = torch.empty(t.tri_edm_workspace_size(n, d, t.BF16X3), dtype=torch.uint8, device=D)
+    t.tri_edm(xd, out, prec=t.BF16X3, workspace=ws, n_flagged=flagged)
+    i = np.arange(1, n, 2)
+    got = out.cpu().numpy()[i * (i + 1) // 2 + i - 1]
+    want = np.sqrt(((x[i].astype(np.float64) - x[i - 1]) ** 2).sum(1))
+    assert flagged.item() >= len(i)
+    assert (got[:30] == 0).all()
+    assert (np.abs(got - want) <= 0.501 * np.spacing(want.astype(np.float32))).all()
+
+
 # --------------------------------------------------------------- AT energy --
 @pytest.mark.parametrize("scale,finite", [(1.0, True), (3e-4, True), (1e-7, False)])
 def test_at_small_products(scale, finite):
