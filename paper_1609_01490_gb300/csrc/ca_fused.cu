@@ -30,6 +30,7 @@
 #include <algorithm>
 
 #include "tri_internal.h"
+#include "pdl.cuh"
 #include "tri_maps.cuh"
 
 using namespace tri;
@@ -139,9 +140,11 @@ __device__ __forceinline__ uint64_t tile_number(int64_t bi, int64_t bj) { return
 // One pass: reads a stored state, takes up to `halo` steps, stores the next.
 template <int MAP>
 __global__ void __launch_bounds__(32, 28)
-    ca_life_run_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, uint32_t n, size_t ld, BlockMap bm,
+    ca_life_run_kernel(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld, BlockMap bm,
                        uint32_t rows, uint32_t steps, int halo, BitStore store)
 {
+    dependents_may_start();
+    wait_for_previous();
     uint32_t bi, bj;
     if (!map_block<MAP>(bm, bi, bj)) return;
     if (bi >= rows) return;  // REC covers a power of two of block rows
@@ -202,6 +205,7 @@ __global__ void __launch_bounds__(32 * RPL)
     ca_life_pack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, uint32_t n, size_t ld, BlockMap bm,
                         uint32_t rows, int halo, BitStore store)
 {
+    dependents_may_start();
     uint32_t bi, bj;
     if (!map_block<MAP>(bm, bi, bj)) return;
     if (bi >= rows) return;
@@ -239,9 +243,10 @@ __global__ void __launch_bounds__(32 * RPL)
 
 template <int MAP>
 __global__ void __launch_bounds__(32 * RPL)
-    ca_life_unpack_kernel(const uint8_t *__restrict__ in, uint8_t *__restrict__ out, uint32_t n, size_t ld,
+    ca_life_unpack_kernel(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld,
                           BlockMap bm, uint32_t rows, int halo, BitStore store)
 {
+    wait_for_previous();
     uint32_t bi, bj;
     if (!map_block<MAP>(bm, bi, bj)) return;
     if (bi >= rows) return;
@@ -315,21 +320,22 @@ int run_fused(const uint8_t *in, uint8_t *out, uint8_t *scratch, uint32_t n, siz
     for (uint32_t p = 0; p < passes && r == TRI_OK; ++p) {
         const uint32_t k = std::min((uint32_t)halo, steps - p * halo);
         r = trihost::map_launches(map, m, [&](auto tag, dim3 g, const BlockMap &bm) -> cudaError_t {
-            ca_life_run_kernel<decltype(tag)::value><<<g, 32, 0, s>>>(at(p), at(p + 1), n, ld, bm, rows, k, halo, store);
-            return cudaGetLastError();
+            return trihost::launch_behind(ca_life_run_kernel<decltype(tag)::value>, g, 32, 0, s, at(p), at(p + 1), n, ld,
+                                          bm, rows, k, halo, store);
         });
     }
     if (r != TRI_OK) return r;
     return trihost::map_launches(map, m, [&](auto tag, dim3 g, const BlockMap &bm) -> cudaError_t {
-        ca_life_unpack_kernel<decltype(tag)::value><<<g, 32 * RPL, 0, s>>>(scratch, out, n, ld, bm, rows, halo, store);
-        return cudaGetLastError();
+        return trihost::launch_behind(ca_life_unpack_kernel<decltype(tag)::value>, g, 32 * RPL, 0, s, scratch, out, n, ld,
+                                      bm, rows, halo, store);
     });
 }
 
 // Passes of 8 steps recompute less halo (1.31 times the tiles' cells against 1.78
 // for passes of 16), but there are twice as many, 5 us apart at the least: 100
-// steps under lambda take, in us (16 / 8 steps a pass), n = 3000: 68 / 92, 6000:
-// 129 / 152, 8000: 175 / 185, 9000: 220 / 215, 12000: 330 / 312, 16384: 576 / 500.
+// steps under lambda take, in us (16 / 8 steps a pass), n = 3000: 61 / 76, 6000:
+// 121 / 148, 8000: 173 / 181, 9000: 199 / 193, 12000: 311 / 276, 16384: 561 / 469
+// (the passes launched behind one another; in stream order 16384: 576 / 500).
 constexpr uint32_t THIN_HALO_N = 8500;
 
 // ------------------------------------------------------- up to 16 steps ----
