@@ -117,8 +117,9 @@ int trihost::edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int ma
         if (st != TRI_OK) return st;
         // few features: the row tile once there are several of its blocks per SM
         // (d = 3, us, 4 x 4 pairs a thread / row tile: n = 65536 1995 / 1209, n = 8000 32.5 /
-        // 24.9, n = 5000 14.4 / 14.1, n = 4000 10.1 / 10.6, n = 2048 4.7 / 7.8)
-        if (d <= (uint32_t)rows::MAX_D && T2(((uint64_t)n + rows::S - 1) / rows::S) >= 800)
+        // 24.9, n = 5000 14.4 / 14.1, n = 4000 10.1 / 10.6, n = 2048 4.7 / 7.8;
+        // d = 8: n = 7000 36.9 / 32.9, n = 6000 28.7 / 28.2, n = 5000 20.6 / 22.6)
+        if (d <= (uint32_t)rows::MAX_D && T2(((uint64_t)n + rows::S - 1) / rows::S) >= (d <= 4 ? 800u : 1200u))
             return launch_rows(x, n, d, out, map, s);
         // more features: 8 x 8 pairs per thread, bound by arithmetic with half the
         // shared-memory reads per pair, once there are three blocks per SM (4 x 4 / 8 x

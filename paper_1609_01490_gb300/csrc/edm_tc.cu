@@ -998,7 +998,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
 // the sum), which round to the FP32 distance that an FP64 sum gives; FP64 itself,
 // at a 64th of FP32's rate, only where a sum leaves [2^-60, 2^100] (there squares
 // may vanish or overflow in FP32).  With 123 equal pairs among N =
-// 12345 points FP64 sums, their warps on two SMs, took 20 us; now 2.
+// 12345 points FP64 sums, their warps on two SMs, took 20 us; now 3 to 5.
 // Takes the list entries appended since the previous call (list entries [*start, count); all of them when start is
 // null).  If the list overflowed, every pair of the packed range [p_begin,
 // p_end) whose stored distance passes a slightly wider version of the flag
