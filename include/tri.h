@@ -85,10 +85,10 @@ typedef enum {
     TRI_FP32 = 0,   /* direct differences in FP32 on CUDA cores */
     TRI_BF16X3 = 1, /* Gram form on tcgen05 tensor cores: rows scaled by powers of
                        two and split into two 16-bit planes (FP16 hi/lo), 3 products,
-                       FP32 accumulation, FP64 recompute of flagged pairs */
+                       FP32 accumulation, direct recompute of flagged pairs */
     TRI_BF16X6 = 2  /* the same with the flag threshold that bounds every result
                        (the accuracy of a hi/mid/lo BF16 split with 6 products):
-                       FP32 accumulation, FP64 recompute of flagged pairs */
+                       FP32 accumulation, direct recompute of flagged pairs */
 } tri_prec;
 
 typedef enum {
@@ -172,16 +172,21 @@ TRI_API int tri_map_first_error(int map, int sqrt_kind, uint64_t n_items, uint64
  *   out[i(i+1)/2 + j] = sqrt(sum_k (x[i][k] - x[j][k])^2), the diagonal 0.
  *   x (device, FP32) row-major [n][d]; out (device, FP32) n(n+1)/2 entries.
  *   prec = TRI_FP32: blocks of rho x rho threads, each thread reg x reg pairs
- *   (reg in {1, 2, 4, 8}, 8 only with rho <= 16; 0 picks 4); each block covers
+ *   (reg in {1, 2, 4, 8}, 8 only with rho <= 16); each block covers
  *   an S x S pair tile, S = rho*reg, placed by `map` (any tri_map).  For reg
- *   >= 2 a thread updates two adjacent columns per f32x2 instruction.  No
- *   workspace.
+ *   >= 2 a thread updates two columns per f32x2 instruction.  reg = 0: the
+ *   library's tile: 128 x 128 tiles stored by rows for d <= 8 and n from about
+ *   5000 (d <= 4) or 6145 on (rho is then only checked), 8 x 8 pairs for more
+ *   features at rho <= 16 once there are 500 such tiles, 4 x 4 otherwise and
+ *   under TRI_MAP_REC.  Every tile gives the same bits and accepts the same
+ *   sizes.  No workspace.
  *   prec = TRI_BF16X3 / TRI_BF16X6: 2 x 2 blocks of 128 x 128 pair tiles per
  *   CTA pair on tcgen05 tensor cores (cta_group::2), placed by
  *   TRI_MAP_LAMBDA or TRI_MAP_BB; rho and reg are ignored;
  *   needs `workspace` of tri_edm_workspace_size bytes (256-byte aligned).
  *   Pairs whose Gram estimate of d^2 falls below tau*(|x_i|^2 + |x_j|^2) are
- *   recomputed in FP64 by direct differences (BF16X6: tau = (2 + 24 c)
+ *   recomputed by direct differences, to the rounding of the FP64 sum
+ *   (BF16X6: tau = (2 + 24 c)
  *   2^-23 / 1.96e-5 for c = ceil(d / 64) K chunks, which bounds every other
  *   distance's relative error by 1e-5; BF16X3: tau = 0.0625, no bound); n_flagged (device uint64,
  *   may be NULL) receives how many were flagged.  If more were flagged than
@@ -222,7 +227,7 @@ TRI_API int tri_edm_workspace_size(uint32_t n, uint32_t d, int prec, size_t *byt
  *     exists so that tests can make those waits run out.  If the two CTAs of
  *     a pair cannot share their tensor-memory address the word becomes
  *     TRI_ECUDA and the pair does no work.
- *   tri_edm_fixup: recomputes the flagged pairs in FP64 by direct differences
+ *   tri_edm_fixup: recomputes the flagged pairs by direct differences
  *     (or, when the list overflowed, every pair whose stored distance passes a
  *     slightly wider flag test) and writes the flag count to *n_flagged
  *     (device uint64, may be NULL).
@@ -238,7 +243,7 @@ TRI_API int tri_edm_fixup(const float *x, uint32_t n, uint32_t d, float *out, in
  * End-to-end EDM from and to host memory (not in the paper, which starts
  * from device-resident points): copies x_host (n x d FP32, row-major) to
  * x_dev, runs tri_edm_prepare, then computes the packed triangle in `bands`
- * row bands (Gram term + FP64 recompute of the band's flagged pairs) and
+ * row bands (Gram term + recompute of the band's flagged pairs) and
  * copies each finished band from out_dev to out_host on a library-owned
  * copy stream while the next band computes, so the device-to-host copy (the
  * bound of this call on a host attached through NVLink-C2C) overlaps the
@@ -342,7 +347,9 @@ TRI_API int tri_edm_batched_partition(const uint32_t *n_k, uint32_t count, uint3
  *   in, out (device uint8, 16-byte aligned) row-major with leading dimension
  *   ld (bytes); ld >= n and ld a multiple of 16; in != out (no aliasing).
  *   map: LAMBDA, LAMBDA_PDELTA, BB, RB or REC.  rho in {8,16,32}: each block
- *   covers a (4 rho) x (4 rho) cell tile.  Conway's rule runs bit-sliced with
+ *   covers a (4 rho) x (4 rho) cell tile, except that Conway's rule takes 128 x
+ *   128-cell tiles from n = 6000 on and other rules 64 x 64 ones at rho = 32 (not
+ *   under REC).  Conway's rule runs bit-sliced with
  *   2 rho threads, each a 32-cell strip of rho/4 consecutive rows held as one
  *   bit per cell (two 16-byte loads per row); other rules run with 4 rho
  *   threads, each a 16-cell strip of byte counters (one 16-byte load per row).
@@ -354,20 +361,24 @@ TRI_API int tri_ca_step(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld,
 
 /*
  * tri_ca_run -- `steps` synchronous steps of the automaton of tri_ca_step,
- * the result in `out`.  Conway's rule at rho = 32 (128 x 128-cell tiles) runs
- * up to 16 steps per pass through memory: one warp per tile reads the tile
- * with a 16-cell halo once, holds it as bits in registers (five region rows
- * per lane, vertical neighbours by warp shuffle), takes the steps there
- * (clearing the cells outside the domain after each) and writes the tile's
- * domain cells once.  Other rules and rho take one tri_ca_step per step.  The
- * result is the same bit for bit as `steps` calls of tri_ca_step.
+ * the result in `out`.  Conway's rule at rho = 32 runs up to 16 steps per pass
+ * through memory: one warp per tile holds the tile and a halo as bits in
+ * registers, takes the steps there (clearing the cells outside the domain
+ * after each) and writes the tile once.  Up to 16 steps run in one pass from
+ * and to bytes (128 x 128-cell tiles, 16-cell halo).  Longer runs pack the grid
+ * into bits, kept in domain cells of out and scratch between passes of 16 steps
+ * (8 from n = 8500 on; 128 x 128-cell regions halo included), and unpack the
+ * last state; grids too small to hold the bits take the one-pass form.  Other
+ * rules and rho take one tri_ca_step per step.  The result is the same bit for
+ * bit as `steps` calls of tri_ca_step.
  *   in (read only), out and scratch (device uint8, 16-byte aligned, row-major
  *   with leading dimension ld as in tri_ca_step): pairwise disjoint.  scratch
  *   holds intermediate states when more than one pass is needed (steps > 16
  *   for the fused form, steps > 1 otherwise) and may be NULL otherwise.  Only
  *   domain cells of out and scratch are written.
  *   map: LAMBDA, LAMBDA_PDELTA, BB, RB or REC; rho in {8,16,32}; steps >= 1.
- *   Issues one launch per pass (REC: one per level and pass) and no host
+ *   Issues one launch per pass, two more for runs of more than 16 steps (REC:
+ *   one per level in place of each), and no host
  *   synchronisation.
  *   Errors: TRI_EINVAL (null, aliasing, bad ld/rho/map/masks, steps = 0,
  *   missing scratch), TRI_ERANGE (REC with a block count that is not a power
@@ -415,8 +426,11 @@ TRI_API int tri_ca_step_rows(const uint8_t *in, uint8_t *out, uint32_t n, size_t
  * takes the same steps reaches the same decisions bit for bit.
  *   centres (device, FP32) row-major [n][dim], dim in {1, 2, 3}; radii
  *   (device, FP32) [n].
- *   map: any tri_map.  rho in {8, 16, 32}; reg in {1, 4, 8} (0 picks 8 for
- *   rho <= 16 and 4 for rho = 32; 8 only with rho <= 16): blocks of rho x rho threads, each thread reg x reg
+ *   map: any tri_map.  rho in {8, 16, 32}; reg in {1, 4, 8} (8 only with rho
+ *   <= 16).  reg = 0, the library's choice, rules out in 2-D and 3-D the pairs
+ *   that surely do not touch by a tensor-core filter on FP16 pairs with a proven
+ *   margin and takes the test above on the rest, in tiles of its own (not under
+ *   REC and UTM); otherwise it is 8 for rho <= 16 and 4 for rho = 32: blocks of rho x rho threads, each thread reg x reg
  *   pairs of an S x S tile, S = rho*reg, whose 2 S spheres are staged in
  *   shared memory (the paper's shared-memory test).  UTM (a thread-space map)
  *   runs one pair per thread from global memory instead; reg is ignored there.

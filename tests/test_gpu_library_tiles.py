@@ -95,6 +95,24 @@ def test_edm_row_tiles(d, n):
             assert bool((buf[:8 + off] == -7.0).all()) and bool((buf[8 + off + size:] == -7.0).all())
 
 
+@pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 8])
+@pytest.mark.parametrize("n", [6145, 6271, 6272])  # one, 127 and 128 rows in the last tile row
+def test_edm_row_tiles_at_chosen_sizes(d, n):
+    # sizes at which tri_edm takes the row tile by itself, for every d <= 8
+    import torch
+    t, D = tri(), dev()
+    x = torch.from_numpy(inputs.edm_normal_points(n, d, seed=n + d)).to(D)
+    size = n * (n + 1) // 2
+    ref = torch.empty(size, device=D)
+    t.tri_edm(x, ref, reg=4)
+    for name in ("LAMBDA", "RB"):
+        for off in range(4):
+            buf = torch.full((size + 16,), -7.0, device=D)
+            t.tri_edm(x, buf[8 + off:8 + off + size], map=getattr(t, "MAP_" + name))
+            assert torch.equal(buf[8 + off:8 + off + size], ref), (name, off)
+            assert bool((buf[:8 + off] == -7.0).all()) and bool((buf[8 + off + size:] == -7.0).all())
+
+
 @pytest.mark.parametrize("d", [9, 16, 33, 100])
 def test_edm_chosen_square_tiles(d):
     # sizes on both sides of the choice between 4 x 4 and 8 x 8 pairs per thread
