@@ -124,7 +124,9 @@ def _hptr(t) -> int:
 
 def _stream(stream) -> int | None:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        # the current stream's handle, without the Stream object around it: the smallest
+        # calls are bound by the host (tri_edm, N = 2048, d = 3: 7.8 us a call with it, 6.2 without)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
 
 
