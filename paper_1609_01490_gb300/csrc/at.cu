@@ -23,9 +23,14 @@ namespace {
 // of the block's setup: the map, the pair quantities and the sums.)
 constexpr int AT_ROWS = 2;
 
+// Four blocks of 512 threads per SM (three where the cubic root needs registers):
+// without the bound the sum took 42 registers, two blocks.  N = 1536, rho = 32, us,
+// table / cubic root / box: unbounded 402 / 446 / 428, three blocks 387 / 414 / 390,
+// four 379 / 433 / 377.
 template <int MAP>
-__global__ void at_kernel(const float *__restrict__ p, uint32_t n, double nu, uint32_t m, uint64_t w0,
-                          uint64_t nblocks, double *__restrict__ partial)
+__global__ void __launch_bounds__(512, MAP == MAP_LAMBDA ? 3 : 4)
+    at_kernel(const float *__restrict__ p, uint32_t n, double nu, uint32_t m, uint64_t w0, uint64_t nblocks,
+              double *__restrict__ partial)
 {
     uint32_t L, R, C;
     if constexpr (MAP == MAP_LAMBDA || MAP == MAP_TET_TABLE) {
@@ -101,7 +106,8 @@ __global__ void at_kernel(const float *__restrict__ p, uint32_t n, double nu, ui
         // The sum over k with the 1 / sqrt that takes subnormal products as zero,
         // keeping the smallest product seen; should one be subnormal (or zero:
         // coincident points), the sum is taken again with rsqrtf, which equals it on
-        // every normal product (N = 1536, rho = 32: 410 us with rsqrtf alone, 402 so).
+        // every normal product (N = 1536, rho = 32: 410 us with rsqrtf alone, 402 so,
+        // before the bound on registers).
         auto sum_over_k = [&](auto exact, float &least) {
             for (t = 0; t + 1 < kend; t += 2) {
                 const f2 b = *reinterpret_cast<const f2 *>(&brow[t]);
