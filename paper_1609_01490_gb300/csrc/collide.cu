@@ -57,27 +57,42 @@ __device__ __forceinline__ void record(const CollideOut &o, uint32_t i, uint32_t
 
 // One S x S pair tile, S = RHO*R: rows i0 = bi S + [0, S), columns
 // j0 = bj S + [0, S).  The 2 S spheres are staged transposed ([coordinate or
-// radius][sphere]), the rows with each value duplicated into both halves of
-// an 8-byte word.  Thread (ty, tx) owns rows ty + u RHO (u < R) and, for
-// R >= 2, the column pairs 2 tx + 2 RHO v + {0, 1} (v < R/2), tested two at a
-// time with f32x2 instructions, whose lanes round exactly as the scalar
-// operations of the reference order do.  The fast pass keeps one word: the
-// AND of the bits of q - s over all the thread's pairs; since q - s rounds to
-// a value >= 0 exactly when q >= s, a clear sign bit means some pair may hit
-// (or some input is NaN).  Only such threads (a few per contact, plus the
-// diagonal, where a sphere meets itself) repeat the packed pass, compare s
-// and q lane by lane and record the valid pairs (i < n, j < i).
-// Padding spheres past n sit at +inf (rows) and -inf (columns), so their
-// tests give s = inf and never flag.  For R = 1 each thread takes the scalar
-// test of its one pair.  Not inlined: every block map calls the same body.
+// radius][sphere]) in dynamic shared memory, the rows with each value duplicated
+// into both halves of an 8-byte word.  Thread (ty, tx) owns rows ty + u RHO (u < R)
+// and, for R >= 2, the column pairs 2 tx + 2 RHO v + {0, 1} (v < R/2), taken two at
+// a time with f32x2 instructions.  Those only rule pairs out: ptxas fuses a packed
+// product into the sum or difference after it, rounding modifiers or not, so a
+// packed form of the exact test misses pairs that touch exactly (s = q).  They form
+// s' - q', s' = s but for at most six roundings and q' from radii widened by
+// 2^-19 of themselves and 2^-73, so that s' < q' wherever s <= q, also where squares
+// vanish in FP32.  A set sign means that the pair may touch (NaNs never do); the
+// thread keeps one bit per row, the OR of its pairs' signs.  Threads with such a row
+// (a few per contact, plus the diagonal, where a sphere meets itself) form s' - q'
+// again there and take the exact test, hit_scalar, of each such pair (i < n, j < i).
+// (With one bit for all its rows a thread repeats 64 pairs for each contact: 65,536
+// spheres in 3-D, reg = 8, took 0.97 ms, now 0.79; on a line 0.57, now 0.46; 9001
+// discs with 400 contacts each 1.01, now 0.41.)  Sums of
+// radii of either sign may cancel and lose the margin, and q' of huge ones is
+// infinite: a tile with a negative radius, or one of 2^62 or more, takes the exact
+// test for all its pairs.  Padding spheres past n sit at +inf (rows) and -inf
+// (columns), where s' = inf.  For R = 1 each thread takes the exact test of its one
+// pair.
+// Not inlined: every block map calls the same body.
+extern __shared__ __align__(16) unsigned char collide_smem[];
+
+template <int RHO, int R, int DIM>
+struct TileBytes {
+    static constexpr int S = RHO * R, ROWS = (DIM + 1) * S * 8, BYTES = ROWS + (DIM + 1) * (S + 2) * 4;
+};
+
 template <int RHO, int R, int DIM>
 __device__ __noinline__ void collide_tile(const float *__restrict__ c, const float *__restrict__ rad, uint32_t n,
                                           uint32_t bi, uint32_t bj, CollideOut o, int tx, int ty)
 {
     constexpr int S = RHO * R;
     constexpr int RC = R == 1 ? 1 : R / 2;
-    __shared__ f2 si[DIM + 1][S];                       // rows, duplicated
-    __shared__ __align__(8) float sj[DIM + 1][S + 2];   // columns
+    f2(*si)[S] = reinterpret_cast<f2(*)[S]>(collide_smem);  // rows, duplicated
+    float(*sj)[S + 2] = reinterpret_cast<float(*)[S + 2]>(collide_smem + TileBytes<RHO, R, DIM>::ROWS);  // columns
     const int tid = ty * RHO + tx;
     const uint64_t i0 = (uint64_t)bi * S, j0 = (uint64_t)bj * S;
     const float inf = __int_as_float(0x7f800000);
@@ -88,14 +103,19 @@ __device__ __noinline__ void collide_tile(const float *__restrict__ c, const flo
         si[k][r] = f2_pack(a, a);
         sj[k][r] = j0 + r < n ? c[j0 * DIM + t] : -inf;
     }
+    bool every = false;  // no margin: all pairs take the exact test
     for (int t = tid; t < S; t += RHO * RHO) {
-        const float a = i0 + t < n ? rad[i0 + t] : 0.0f;
+        float a = i0 + t < n ? rad[i0 + t] : 0.0f, b = j0 + t < n ? rad[j0 + t] : 0.0f;
+        every = every || fminf(a, b) < 0.0f || fmaxf(a, b) >= 4.6116860e18f;
+        if constexpr (R > 1) {
+            a = fmaf(a, 1.0000019f, 1.0587912e-22f);
+            b = fmaf(b, 1.0000019f, 1.0587912e-22f);
+        }
         si[DIM][t] = f2_pack(a, a);
-        sj[DIM][t] = j0 + t < n ? rad[j0 + t] : 0.0f;
+        sj[DIM][t] = b;
     }
-    __syncthreads();
-
     if constexpr (R == 1) {
+        __syncthreads();
         float a[DIM + 1], b[DIM + 1], dummy;
 #pragma unroll
         for (int k = 0; k <= DIM; ++k) {
@@ -106,56 +126,79 @@ __device__ __noinline__ void collide_tile(const float *__restrict__ c, const flo
         if (hit_scalar<DIM>(a, b) && i < n && j < i) record(o, (uint32_t)i, (uint32_t)j);
         return;
     } else {
+        every = __syncthreads_or(every);
         f2 b2[RC][DIM + 1];
 #pragma unroll
         for (int v = 0; v < RC; ++v)
 #pragma unroll
             for (int k = 0; k <= DIM; ++k) b2[v][k] = *reinterpret_cast<const f2 *>(&sj[k][2 * tx + 2 * RHO * v]);
-        // s and q of the column pair v for row values a2, in the reference order
-        auto test = [&](const f2 *a2, int v, f2 &s, f2 &q) {
+        // s' - q' of the column pair v for row values a2: sign set if the pair may touch
+        auto filter = [&](const f2 *a2, int v) {
+            f2 s;
 #pragma unroll
             for (int k = 0; k < DIM; ++k) {
                 const f2 dk = f2_sub(a2[k], b2[v][k]);
-                s = k == 0 ? f2_mul(dk, dk) : f2_add(s, f2_mul(dk, dk));
+                s = k == 0 ? f2_mul(dk, dk) : f2_fma(dk, dk, s);
             }
             const f2 rr = f2_add(a2[DIM], b2[v][DIM]);
-            q = f2_mul(rr, rr);
+            return f2_sub(s, f2_mul(rr, rr));
         };
-        uint32_t acc = 0xFFFFFFFFu;
+        uint32_t near = 0;  // bit R - 1 - u: some pair of row u may touch
 #pragma unroll
         for (int u = 0; u < R; ++u) {
             f2 a2[DIM + 1];
 #pragma unroll
             for (int k = 0; k <= DIM; ++k) a2[k] = si[k][ty + u * RHO];
+            uint32_t acc = 0;
 #pragma unroll
             for (int v = 0; v < RC; ++v) {
-                f2 s, q;
-                test(a2, v, s, q);
-                const f2 d = f2_sub(q, s);
-                acc &= (uint32_t)d & (uint32_t)(d >> 32);
+                const f2 e = filter(a2, v);
+                acc |= (uint32_t)e | (uint32_t)(e >> 32);
             }
+            near = __funnelshift_l(acc, near, 1);
         }
-        if ((int)acc < 0) return;
-        // some pair may hit: the same tests again, decided lane by lane
-#pragma unroll 1
-        for (int u = 0; u < R; ++u) {
+        if (every) near = (1u << R) - 1u;
+        // the exact test of the pairs that may touch.  Without a list one addition per
+        // row and thread, and one of the thread's pairs.
+        uint32_t found = 0;
+        for (; near; near &= near - 1) {
+            const int u = R - __ffs(near);
             const uint64_t i = i0 + ty + u * RHO;
-            if (i >= n) break;
+            if (i >= n) continue;
+            uint32_t row = 0;
             f2 a2[DIM + 1];
 #pragma unroll
             for (int k = 0; k <= DIM; ++k) a2[k] = si[k][ty + u * RHO];
 #pragma unroll
             for (int v = 0; v < RC; ++v) {
-                f2 s, q;
-                test(a2, v, s, q);
-                float s0, s1, q0, q1;
-                f2_unpack(s, s0, s1);
-                f2_unpack(q, q0, q1);
+                const f2 e = filter(a2, v);
                 const uint64_t j = j0 + 2 * tx + 2 * RHO * v;
-                if (s0 <= q0 && j < i) record(o, (uint32_t)i, (uint32_t)j);
-                if (s1 <= q1 && j + 1 < i) record(o, (uint32_t)i, (uint32_t)(j + 1));
+                const bool lo = ((int)(uint32_t)e < 0 || every) && j < i;
+                const bool hi = ((int)(uint32_t)(e >> 32) < 0 || every) && j + 1 < i;
+                if (!lo && !hi) continue;
+                float a[DIM + 1], b0[DIM + 1], b1[DIM + 1], dummy;
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) {
+                    f2_unpack(a2[k], a[k], dummy);
+                    f2_unpack(b2[v][k], b0[k], b1[k]);
+                }
+                a[DIM] = rad[i];
+                b0[DIM] = lo ? rad[j] : 0.0f;
+                b1[DIM] = hi ? rad[j + 1] : 0.0f;
+                const bool h0 = lo && hit_scalar<DIM>(a, b0), h1 = hi && hit_scalar<DIM>(a, b1);
+                if (o.pairs) {
+                    if (h0) record(o, (uint32_t)i, (uint32_t)j);
+                    if (h1) record(o, (uint32_t)i, (uint32_t)(j + 1));
+                } else {
+                    row += (h0 ? 1u : 0u) + (h1 ? 1u : 0u);
+                    if (o.count && h0) atomicAdd(o.count + j, 1u);
+                    if (o.count && h1) atomicAdd(o.count + j + 1, 1u);
+                }
             }
+            found += row;
+            if (o.count && row) atomicAdd(o.count + i, row);
         }
+        if (found) atomicAdd(o.n_pairs, (unsigned long long)found);
     }
 }
 
@@ -180,20 +223,17 @@ __device__ __noinline__ void collide_tile(const float *__restrict__ c, const flo
 // mma.sync m16n8k16 leaves each thread its results in registers, so the test of
 // 512 pairs per warp is 4 instructions on the tensor core, 8 three-input ANDs
 // and a vote, against about 50 packed FP32 instructions.
-// 65,536 spheres in 3-D take 218 us against 970 with the packed FP32 tile,
-// 9001 in 2-D 18.6 against 48.  The tensor core bounds it (one m16n8k16 per SM
+// 65,536 spheres in 3-D take 215 us against 786 with the packed FP32 tile,
+// 9001 in 2-D 13 against 29.  The tensor core bounds it (one m16n8k16 per SM
 // takes 1.04 ns: 115 us), then the staging of each block's spheres.
 // The margin is 3e-5 of the block's squared extent, so it flags few pairs unless
 // most spheres crowd into a small part of that extent (or meet many others):
 // each warp counts the flags of its first 512 pairs, and a block that finds more
 // than 1 in 128 runs the packed FP32 tile instead (not where values are infinite
-// or squares may overflow or vanish: that tile's sign test and packed arithmetic
-// are not exact there, the one-pair test is).  On a line (1-D) the margin
-// alone flags 1 in 180 pairs (0.63 against 0.59 ms): those keep the FP32 tile.
+// or squares may overflow or vanish).  On a line (1-D) the margin
+// alone flags 1 in 180 pairs (0.63 ms against 0.46): those keep the FP32 tile.
 constexpr int MMA_THREADS = 256;
-#ifndef MMA_BLOCKS
-#define MMA_BLOCKS 4
-#endif
+constexpr int MMA_BLOCKS = 4;
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
 __device__ __forceinline__ float redux_min(float v)
@@ -247,10 +287,9 @@ __device__ __noinline__ void collide_tile_mma(const float *__restrict__ c, const
 {
     constexpr int NT = MMA_THREADS, NW = NT / 32, PER = 2 * S / NT;  // spheres staged per thread
     static_assert(S % 64 == 0 && S / 64 <= NW && PER >= 1, "row groups of 64 rows");
-    extern __shared__ __align__(16) unsigned char mma_smem[];
     // operand records (16 halves) of the S rows and S columns, then the spheres themselves
-    uint4 *rec = reinterpret_cast<uint4 *>(mma_smem);
-    float4 *pos = reinterpret_cast<float4 *>(mma_smem + 2 * S * 32);
+    uint4 *rec = reinterpret_cast<uint4 *>(collide_smem);
+    float4 *pos = reinterpret_cast<float4 *>(collide_smem + 2 * S * 32);
     __shared__ float s_red[NW][2 * DIM + 1];
     __shared__ uint32_t s_flags[NW];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -538,7 +577,7 @@ int launch_dim(const float *c, const float *rad, uint32_t n, int map, uint32_t r
         constexpr int MAP = decltype(tag)::value;
 #define TRI_C(RH, RG)                                                                                          \
     if (rho == RH && reg == RG) {                                                                              \
-        collide_kernel<MAP, RH, RG, DIM><<<g, dim3(RH, RH), 0, s>>>(c, rad, n, o, bm);                         \
+        collide_kernel<MAP, RH, RG, DIM><<<g, dim3(RH, RH), TileBytes<RH, RG, DIM>::BYTES, s>>>(c, rad, n, o, bm); \
         return cudaGetLastError();                                                                             \
     }
         TRI_C(8, 1) TRI_C(8, 4) TRI_C(8, 8) TRI_C(16, 1) TRI_C(16, 4) TRI_C(16, 8) TRI_C(32, 1) TRI_C(32, 4)

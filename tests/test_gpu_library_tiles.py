@@ -75,6 +75,71 @@ def test_collide_filter_scales(orc, case):
         _check_collide(orc, c, r)
 
 
+@pytest.mark.parametrize("dim", [1, 2, 3])
+@pytest.mark.parametrize("reg", [0, 4, 8])
+def test_collide_exact_touch(orc, dim, reg):
+    """Pairs that touch exactly, s = q after rounding: their squares round up and
+    down alike.  Packed products fused into the next sum would miss half of them."""
+    import torch
+    t, D, n = tri(), dev(), 1400
+    rng = np.random.default_rng(dim)
+    gap = rng.integers(1 << 12, 1 << 14, n // 2) * 2.0 ** -12  # 13-bit gaps: differences and sums are exact
+    c = np.zeros((n, dim))
+    c[::2, 0] = 5.0 * np.arange(n // 2)
+    c[1::2, 0] = c[::2, 0] + gap
+    r = np.repeat(gap / 2, 2)
+    order = np.concatenate([np.arange(0, n, 2), np.arange(1, n, 2)])  # partners far apart, no diagonal pair beside them
+    c, r = c[order], r[order]
+    scale = np.float32(1.1)  # 24-bit values, each pair still at equal rounded distance and radius sum or apart
+    for c32, r32 in ((c.astype(np.float32), r.astype(np.float32)),
+                     ((c * (2 ** 12 + 1)).astype(np.float32) * scale, (r * (2 ** 12 + 1)).astype(np.float32) * scale)):
+        cnt_ref, pi, _ = orc.collide_counts(c32, r32)
+        npairs = torch.zeros(1, dtype=torch.int64, device=D)
+        count = torch.zeros(n, dtype=torch.int32, device=D)
+        t.tri_collide(torch.from_numpy(c32).to(D), torch.from_numpy(r32).to(D), npairs, count=count, reg=reg)
+        assert npairs.item() == len(pi)
+        np.testing.assert_array_equal(count.cpu().numpy().astype(np.uint32), cnt_ref)
+
+
+@pytest.mark.parametrize("reg", [4, 8])
+@pytest.mark.parametrize("e", [-70, -66, 0, 61, 80])
+def test_collide_packed_tile_scales(orc, reg, e):
+    # squares that vanish or overflow in FP32, and radii of either sign, through the
+    # packed tile itself
+    import torch
+    t, D, n = tri(), dev(), 500
+    for dim in (2, 3):
+        c, r = inputs.spheres(n, dim, kappa=4.0, seed=n + dim)
+        c, r = np.ldexp(c, e).astype(np.float32), np.ldexp(r, e).astype(np.float32)
+        if e == 0:
+            r[::3] *= np.float32(-0.75)
+        r[7] = np.inf
+        with np.errstate(all="ignore"):
+            cnt_ref, pi, _ = orc.collide_counts(c, r)
+        npairs = torch.zeros(1, dtype=torch.int64, device=D)
+        count = torch.zeros(n, dtype=torch.int32, device=D)
+        t.tri_collide(torch.from_numpy(c).to(D), torch.from_numpy(r).to(D), npairs, count=count, reg=reg)
+        assert npairs.item() == len(pi)
+        np.testing.assert_array_equal(count.cpu().numpy().astype(np.uint32), cnt_ref)
+
+
+@pytest.mark.parametrize("n", [6401, 18001])  # 256- and 512-sphere tiles, ragged ends
+@pytest.mark.parametrize("case", ["crowd", "tiny", "special"])
+def test_collide_filter_gives_up_at_larger_tiles(orc, n, case):
+    # the packed FP32 tiles inside a larger block: the skips above the diagonal and past n
+    c, r = inputs.spheres(n, 3, kappa=4.0, seed=n)
+    c, r = c.copy(), r.copy()
+    if case == "crowd":
+        c[::97] *= np.float32(4000.0)
+    elif case == "tiny":
+        c, r = np.ldexp(c, -70).astype(np.float32), np.ldexp(r, -70).astype(np.float32)
+    else:
+        c[::3, 1] = np.nan
+        c[5, 0], r[33], r[n - 1] = np.inf, np.inf, np.nan
+    with np.errstate(all="ignore"):
+        _check_collide(orc, c, r, ("LAMBDA", "RB"))
+
+
 # ------------------------------------------------------------ FP32 distances --
 @pytest.mark.parametrize("d", [1, 2, 3, 4, 5, 8])
 @pytest.mark.parametrize("n", [1, 3, 125, 126, 127, 128, 129, 256, 383, 700])
