@@ -224,13 +224,14 @@ __device__ __noinline__ void collide_tile(const float *__restrict__ c, const flo
 // 512 pairs per warp is 4 instructions on the tensor core, 8 three-input ANDs
 // and a vote, against about 50 packed FP32 instructions.
 // 65,536 spheres in 3-D take 215 us against 786 with the packed FP32 tile,
-// 9001 in 2-D 13 against 29.  The tensor core bounds it (one m16n8k16 per SM
+// 9001 in 2-D 13 against 19.  The tensor core bounds it (one m16n8k16 per SM
 // takes 1.04 ns: 115 us), then the staging of each block's spheres.
 // The margin is 3e-5 of the block's squared extent, so it flags few pairs unless
 // most spheres crowd into a small part of that extent (or meet many others):
 // each warp counts the flags of its first 512 pairs, and a block that finds more
-// than 1 in 128 runs the packed FP32 tile instead (not where values are infinite
-// or squares may overflow or vanish).  On a line (1-D) the margin
+// than 1 in 128 runs the packed FP32 tile instead: 1 in 4 where infinities or NaNs
+// flag whole rows (18,000 spheres, one infinite radius: 33 us pair by pair, 104
+// packed; every third a NaN: 283 and 122).  On a line (1-D) the margin
 // alone flags 1 in 180 pairs (0.63 ms against 0.46): those keep the FP32 tile.
 constexpr int MMA_THREADS = 256;
 constexpr int MMA_BLOCKS = 4;
@@ -426,7 +427,7 @@ __device__ __noinline__ void collide_tile_mma(const float *__restrict__ c, const
 #pragma unroll
     for (int w = 0; w < NW; ++w) total += s_flags[w];
     wait_for_previous();  // the outputs are zeroed from here on
-    if (total > NW * 512 / 128 && usable && !odd) {
+    if (total > (odd ? NW * 512 / 4 : NW * 512 / 128)) {
         constexpr int Q = S / 128;  // packed FP32 tiles a side
         for (int w = 0; w < Q * Q; ++w) {
             const uint32_t ti = bi * Q + w / Q, tj = bj * Q + w % Q;
