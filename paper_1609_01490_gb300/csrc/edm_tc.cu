@@ -835,12 +835,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
             for (int v = 0; v < NCH / 2; ++v) {
                 const uint32_t u = 2 * v + (lane >> 4);
                 const uint32_t ii = a * TILE + (grp + NG * u) * EPI_ROWS + (lane & 15);
-                pfr[v] = ii < g.n ? __ldg(g.norms + ii) : 0.0f;
-                pfs[v] = ii < g.n ? __ldg(g.scales + ii) : 0.0f;
+                pfr[v] = ii < g.n ? g.norms[ii] : 0.0f;
+                pfs[v] = ii < g.n ? g.scales[ii] : 0.0f;
             }
             const uint32_t jj = b * TILE + q * 32 + lane;
-            pfj = jj < g.n ? __ldg(g.norms + jj) : 0.0f;
-            pfjs = jj < g.n ? __ldg(g.scales + jj) : 0.0f;
+            pfj = jj < g.n ? g.norms[jj] : 0.0f;
+            pfjs = jj < g.n ? g.scales[jj] : 0.0f;
         };
         uint32_t acc = 0, acc_phase = 0, nbuf = 0, k = 0;
         auto fail = [&]() {

@@ -6,10 +6,12 @@
 // 9001 discs takes 18.6 us (21.5 in stream order), a cost-model step 18.8 (20.4).
 // A waiting block keeps its place: the blocks of the second kernel gather on the
 // SMs that the first leaves early, so work that only a few blocks have is spread.
-// Only between two kernels of one call on one stream: the first is launched in
-// the ordinary way, so that it follows everything before it in the stream.
-// A kernel launched so never reads the first one's results through const
-// __restrict__ pointers: such loads may be moved ahead of the wait.
+// Only between kernels of one call on one stream: the first is launched in the
+// ordinary way, so that it follows everything before it in the stream, and each of the
+// others waits before it touches anything that an earlier one writes or reads, so
+// that a chain of them keeps its order.  A kernel launched so never reads an earlier
+// one's results through const __restrict__ pointers or __ldg: such loads may be moved
+// ahead of the wait, or come from a cache filled before it.
 #pragma once
 
 #include <cuda_runtime.h>
