@@ -80,6 +80,10 @@ constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr int MAX_STAGES = 12;             // B ring depth cap (16 KB stages)
 
 constexpr float TAU_X3 = 0.0625f;  // flag threshold of TRI_BF16X3 (no bound asked for)
+// A pair with d^2 <= tau (|x_i|^2 + |x_j|^2) + TINY is flagged: below 2^-116 the
+// squares' own underflow (320 roundings of 2^-150 at most) and a root that takes
+// subnormal numbers as zero would show; above it they are 2^-25 of d^2.
+constexpr float TINY = 1.2037062e-35f;  // 2^-116
 
 // Flag threshold of TRI_BF16X6 with nkc 64-wide K chunks.  The Gram term's
 // error is at most 2^-21 (both rows' planes, 2^-23 each, and the dropped
@@ -898,7 +902,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         const float *un = rn + u * EPI_ROWS, *us = rs + u * EPI_ROWS;
                         // two rows per instruction: d2 = |x_i|^2 + |x_j|^2 - 2 x_i.x_j;
                         // one test per chunk for a pair with d2 <= tau (|x_i|^2 +
-                        // |x_j|^2) (cancellation, the diagonal, or padding).  The
+                        // |x_j|^2) + TINY (cancellation, the diagonal, or padding).  The
                         // scales go in one after the other: each product stays in
                         // FP32's range wherever the norms do.
                         float dv[EPI_ROWS], d2v[EPI_ROWS], w[EPI_ROWS];
@@ -921,11 +925,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         float worst = 1.0f;
 #pragma unroll
                         for (int k = 0; k < EPI_ROWS; k += 2) worst = min3(worst, w[k], w[k + 1]);
-                        if (worst <= 0.0f) {
+                        if (worst <= TINY) {
 #pragma unroll
                             for (int k = 0; k < EPI_ROWS; ++k) {
                                 const float d2 = d2v[k];
-                                if (d2 <= tau * (un[k] + nj)) {
+                                if (d2 <= fmaf(tau, un[k] + nj, TINY)) {
                                     const uint32_t i = i0 + k;
                                     if (i < g.n && j < i) {
                                         const unsigned long long slot = atomicAdd(g.flag_count, 1ull);
@@ -1090,7 +1094,7 @@ __global__ void fixup_kernel(const float *__restrict__ x, uint32_t d, float *__r
             lambda_diag<TRI_SQRT_X>((uint32_t)p, i, j);
             if (i == j) continue;
             const float v = out[p];
-            if (v * v < wide * (norms[i] + norms[j])) recompute(i, j);
+            if (v * v <= fmaf(wide, norms[i] + norms[j], 2.0f * TINY)) recompute(i, j);
         }
     }
 }

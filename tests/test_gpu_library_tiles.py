@@ -334,3 +334,38 @@ def test_at_small_products(scale, finite):
         assert abs(energy.item() - want) <= 2e-5 * want
     else:
         assert energy.item() == float("inf")
+
+
+# ------------------------------------------- tensor-core distances, accuracy --
+def _tc_edm(x, prec):
+    import torch
+    t, n = tri(), x.shape[0]
+    out = torch.empty(n * (n + 1) // 2, device=x.device)
+    ws = torch.empty(t.tri_edm_workspace_size(n, x.shape[1], prec), dtype=torch.uint8, device=x.device)
+    t.tri_edm(x, out, prec=prec, workspace=ws)
+    return out
+
+
+def _packed64(x):
+    """Packed lower triangle of distances by direct differences, in 64 bits."""
+    import torch
+    n, xd = x.shape[0], x.double()
+    ref = torch.zeros(n, n, dtype=torch.float64, device=x.device)
+    for k in range(x.shape[1]):
+        df = xd[:, k, None] - xd[None, :, k]
+        ref.addcmul_(df, df)
+    return ref.sqrt_()[torch.tril(torch.ones_like(ref, dtype=torch.bool))]
+
+
+@pytest.mark.parametrize("prec", ["BF16X6", "BF16X3"])
+@pytest.mark.parametrize("n", [300, 1500])  # the second has more pairs than the list of flagged ones holds
+@pytest.mark.parametrize("e", [-25, -24, -23, -22, -21, -20, -19])
+def test_tc_edm_tiny_rows(prec, n, e):
+    """Squares at the edge of FP32's range and below it: flagged and recomputed, so
+    within 1e-5 like all others."""
+    import torch
+    g = torch.Generator(device=dev()).manual_seed(n)
+    for d in (2, 64):
+        x = (torch.randn(n, d, generator=g, device=dev()).double() * 10.0 ** e).float()
+        got, ref = _tc_edm(x, getattr(tri(), prec)).double(), _packed64(x)
+        assert bool(((got - ref).abs() <= 1e-5 * ref).all()), d
