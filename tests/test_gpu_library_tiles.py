@@ -369,3 +369,15 @@ def test_tc_edm_tiny_rows(prec, n, e):
         x = (torch.randn(n, d, generator=g, device=dev()).double() * 10.0 ** e).float()
         got, ref = _tc_edm(x, getattr(tri(), prec)).double(), _packed64(x)
         assert bool(((got - ref).abs() <= 1e-5 * ref).all()), d
+
+
+def test_tc_edm_recompute_rounds_as_fp64():
+    """Recomputed pairs are FP64 sums rounded once: half an ulp and, for the sum's own
+    rounding of at most 64 steps, 2^-24 of one."""
+    import torch
+    D = dev()
+    for seed in range(6):
+        x = 100.0 + torch.randn(1400, 64, generator=torch.Generator(device=D).manual_seed(seed), device=D)
+        got, ref = _tc_edm(x, tri().BF16X3).double(), _packed64(x)
+        ulp = torch.exp2(torch.floor(torch.log2(ref.clamp_min(1e-30))) - 23)
+        assert bool(((got - ref).abs() <= (0.5 + 2.0 ** -24) * ulp).all()), seed
