@@ -10,11 +10,10 @@
 // hi.lo', lo.hi' and drops lo.lo', below 2^-22 |x||y|; every FP16 x FP16 product
 // is exact in FP32, and the epilogue takes the scales out again (exact powers
 // of two).  Both tensor-core precisions use this split and differ in the flag
-// threshold.  A BF16 split needs three planes
-// and six products for the same bits.  At N = 65536, d = 128 that took 2.18 ms
-// a call against 1.80 ms here (1.78 ms of it the six products' tensor time at
-// the measured peak), and its relative error against 64 bits was 7.2e-8 against
-// 4.8e-8: the planes' rounding costs less than twice the accumulation steps.
+// threshold.  A BF16 split takes three planes and six products to hold every bit of
+// an input: at N = 65536, d = 128 2.18 ms a call against 1.81 ms here (1.78 ms of it
+// the six products' tensor time at the measured peak), with a relative error against
+// 64 bits of 7.2e-8 against 4.1e-8: each product less is less truncation.
 // A pair whose estimate falls below tau (|x_i|^2 + |x_j|^2) has lost
 // too many digits to cancellation and is flagged; a second kernel recomputes
 // flagged pairs by direct differences (the paper's definition).
@@ -87,10 +86,10 @@ constexpr float TINY = 1.2037062e-35f;  // 2^-116
 
 // Flag threshold of TRI_BF16X6 with nkc 64-wide K chunks.  The Gram term's
 // error is at most 2^-21 (both rows' planes, 2^-23 each, and the dropped
-// product, 2^-22) plus 2^-23 per FP32 accumulation step (12 MMAs of K = 16 per
-// chunk: 3 plane products x 4) of sum_k |x_ik x_jk| <= (|x_i|^2 + |x_j|^2) / 2,
+// product, 2^-22) plus 2^-23 per FP32 accumulation step at full size (4 MMAs of K =
+// 16 per chunk, hi.hi', after the small terms) of sum_k |x_ik x_jk| <= (|x_i|^2 + |x_j|^2) / 2,
 // so with the norms' and the final combination's roundings |error of d^2| <=
-// (5 + 12 nkc) 2^-23 (|x_i|^2 + |x_j|^2).  The relative error of d is about
+// (6 + 4 nkc) 2^-23 (|x_i|^2 + |x_j|^2).  The relative error of d is about
 // half that of d^2, and the square root adds up to ~1.5e-7.  tau keeps the
 // larger value (2 + 24 nkc) 2^-23 / (2 (1e-5 - 2e-7)) of a split with 24 steps
 // per chunk, so that the same pairs are flagged: a pair with d^2 > tau
@@ -461,8 +460,12 @@ __device__ __forceinline__ bool unit_of(uint64_t u, uint32_t mb, uint32_t &R, ui
     }
 }
 
-// The split keeps the products of row plane pa and column plane pb with
-// pa + pb <= P - 1: hi.hi, lo.hi and hi.lo.
+// The split keeps hi.lo', lo.hi' and hi.hi'.  Every MMA truncates its sum to FP32, so
+// the order matters: the hi.lo' of all chunks, then the lo.hi', while the sum is 2^-11
+// of its final size, then the hi.hi'.  With the three products of each chunk together,
+// the FP32 steps at full size are three times as many.  Relative error against 64 bits,
+// root mean square / largest, in that order and so: N(0,1)^100 points 4.4e-8, 3.3e-8;
+// U[0,1)^256 2.7e-6 / 6.9e-6, 1.7e-6 / 3.8e-6 (two BF16 planes: 1.6e-6 / 6.5e-6).
 
 // Barrier among the `count` threads of one epilogue row group (ids 1..).
 __device__ __forceinline__ void named_sync(uint32_t id, uint32_t count)
@@ -644,7 +647,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     // 256x256x16 pair MMA takes about 136 cycles on each SM, and any longer
     // gap in the issue stream leaves the tensor pipes idle.  Each stage holds
     // one plane of one 64-wide K chunk of a CTA's column block: the MMA thread
-    // waits once per 4 (P - pb) MMAs for column plane pb.
+    // waits once per stage; it issues four MMAs for a lo plane and eight for a hi
+    // plane, which stays in its stage until its second four.
     if (warp == 0) {
         // ------------------------------------------------ TMA producer (both CTAs)
         if (lane == 0 && run) {
@@ -693,19 +697,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                     ++a_loads;
                     a_row = R;
                 }
-                for (uint32_t kc = 0; kc < g.nkc && ok; ++kc) {
-                    for (int pl = 0; pl < P; ++pl) {
-                        if (!mbar_wait(b_emptyB + 8 * stage, b_phase ^ 1, &s_abort, wl)) {
-                            ok = false;
-                            break;
-                        }
-                        if (leader) mbar_expect_tx(b_fullB + 8 * stage, 2 * stage_bytes);
-                        tma_load_3d_pair(sB + stage * CHUNK_BYTES, &tmap, L_fullB + 8 * stage, kc * KCH, cb * TILE, pl);
-                        ++loads;
-                        if (++stage == g.stages) {
-                            stage = 0;
-                            b_phase ^= 1;
-                        }
+                // the lo planes of all chunks, then the hi planes
+                for (uint32_t q = 0; q < 2 * g.nkc; ++q) {
+                    const bool lo = q < g.nkc;
+                    if (!mbar_wait(b_emptyB + 8 * stage, b_phase ^ 1, &s_abort, wl)) {
+                        ok = false;
+                        break;
+                    }
+                    if (leader) mbar_expect_tx(b_fullB + 8 * stage, 2 * stage_bytes);
+                    tma_load_3d_pair(sB + stage * CHUNK_BYTES, &tmap, L_fullB + 8 * stage, (lo ? q : q - g.nkc) * KCH,
+                                     cb * TILE, lo ? 1 : 0);
+                    ++loads;
+                    if (++stage == g.stages) {
+                        stage = 0;
+                        b_phase ^= 1;
                     }
                 }
                 if (!ok) break;
@@ -777,29 +782,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                 }
                 tc_fence_after();
                 const uint32_t d_tmem = tmem + acc * (2 * TILE);  // 256 columns per accumulator
-                for (uint32_t kc = 0; kc < g.nkc && ok; ++kc) {
-                    const uint64_t a_desc = a_desc0 + kc * P * CH16;
+                // the column blocks are the M operand: TMEM lane = output column; +2 per
+                // 16-element K step (32 bytes in 16-byte units)
+                auto products = [&](uint32_t st, uint64_t a_desc, bool first) {
+                    const uint64_t b_desc = b_desc0 + st * CH16;
 #pragma unroll
-                    for (int pb = 0; pb < P; ++pb) {
+                    for (int kk = 0; kk < KCH / 16; ++kk)
+                        umma2_f16(d_tmem, b_desc + 2 * kk, a_desc + 2 * kk, kk == 0 && first ? 0u : 1u);
+                };
+                auto advance = [&]() {
+                    if (++stage == g.stages) {
+                        stage = 0;
+                        b_phase ^= 1;
+                    }
+                };
+                // lo planes of the columns with hi planes of the rows
+                for (uint32_t kc = 0; kc < g.nkc; ++kc) {
+                    if (!mbar_wait(b_fullB + 8 * stage, b_phase, &s_abort, wl)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    products(stage, a_desc0 + kc * P * CH16, kc == 0);
+                    umma2_commit_both(b_emptyB + 8 * stage);  // stage free (both CTAs) when these MMAs finish
+                    advance();
+                }
+                // hi planes of the columns, as many chunks at a time as the ring holds:
+                // with the lo planes of the rows, then, still in their stages, with the hi planes
+                for (uint32_t k0 = 0; k0 < g.nkc && ok; k0 += g.stages) {
+                    const uint32_t k1 = min(g.nkc, k0 + g.stages);
+                    uint32_t held = stage;
+                    for (uint32_t kc = k0; kc < k1; ++kc) {
                         if (!mbar_wait(b_fullB + 8 * stage, b_phase, &s_abort, wl)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        const uint64_t b_desc = b_desc0 + stage * CH16;
-#pragma unroll
-                        for (int pa = 0; pa + pb < P; ++pa)
-#pragma unroll
-                            for (int kk = 0; kk < KCH / 16; ++kk)
-                                // the column blocks are the M operand: TMEM lane = output
-                                // column; +2 per 16-element K step (32 bytes in 16-byte units)
-                                umma2_f16(d_tmem, b_desc + 2 * kk, a_desc + pa * CH16 + 2 * kk,
-                                           (kc | pb | pa | kk) ? 1u : 0u);
-                        umma2_commit_both(b_emptyB + 8 * stage);  // stage free (both CTAs) when these MMAs finish
-                        if (++stage == g.stages) {
-                            stage = 0;
-                            b_phase ^= 1;
-                        }
+                        products(stage, a_desc0 + (kc * P + 1) * CH16, false);
+                        advance();
+                    }
+                    for (uint32_t kc = k0; kc < k1 && ok; ++kc) {
+                        products(held, a_desc0 + kc * P * CH16, false);
+                        umma2_commit_both(b_emptyB + 8 * held);
+                        if (++held == g.stages) held = 0;
                     }
                 }
                 if (!ok) break;
@@ -946,13 +971,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
                         // same 16 rows; a barrier before their stores keeps them
                         // writing the same rows at the same time, so the partly
                         // written 32-byte sectors at the quarters' edges meet in L2
-                        // soon after each other (BF16X6, N = 65536, d = 128: 2.24 ms
-                        // with one barrier per unit, 2.19 per tile, 2.09 per 16
-                        // rows, 2.09 per 8, 2.14 per 4).  Staging whole row segments
-                        // through shared memory competes with the tensor core's
-                        // operand reads: BF16X6 2.51 ms, BF16X3 2.42 ms against
-                        // 1.95 ms direct; assembling only the 32-byte sectors that
-                        // straddle two quarters of a row, 2.63 ms.
+                        // soon after each other (taken with six BF16 products, N =
+                        // 65536, d = 128: 2.24 ms with one barrier per unit, 2.19 per
+                        // tile, 2.09 per 16 rows, 2.09 per 8, 2.14 per 4).  Staging
+                        // whole row segments through shared memory competes with the
+                        // tensor core's operand reads (then 2.51 ms; with three
+                        // products 2.42 against 1.95 direct); assembling only the
+                        // 32-byte sectors that straddle two quarters of a row, 2.63 ms.
                         named_sync(1 + grp, 128);
                         float *row = g.out + T2(i0) + j;  // row i0, column j
                         if (bi != bj && (bi + 1) * TILE <= g.n) {

@@ -381,3 +381,16 @@ def test_tc_edm_recompute_rounds_as_fp64():
         got, ref = _tc_edm(x, tri().BF16X3).double(), _packed64(x)
         ulp = torch.exp2(torch.floor(torch.log2(ref.clamp_min(1e-30))) - 23)
         assert bool(((got - ref).abs() <= (0.5 + 2.0 ** -24) * ulp).all()), seed
+
+
+@pytest.mark.parametrize("d,most", [(224, 5.29e-6), (256, 5.23e-6), (320, 6.02e-6)])
+def test_tc_edm_sum_order(d, most):
+    """Uniform points, whose inner products grow with every step, so that the sums'
+    truncation shows: no further off than the two-plane BF16 split that this one
+    replaced, whose largest relative errors on these points are given."""
+    import torch
+    n = 1999
+    x = torch.rand(n, d, generator=torch.Generator(device=dev()).manual_seed(1000 * d + n + 2), device=dev())
+    got, ref = _tc_edm(x, tri().BF16X3).double(), _packed64(x)
+    off = ref > 0
+    assert float(((got - ref).abs() / ref)[off].max()) <= most
