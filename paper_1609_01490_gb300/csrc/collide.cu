@@ -13,6 +13,7 @@
 
 #include "f32x2.cuh"
 #include "pdl.cuh"
+#include "tri_internal.h"
 #include "tri_maps.cuh"
 
 using namespace tri;
@@ -500,8 +501,7 @@ int launch_mma(const float *c, const float *rad, uint32_t n, int map, CollideOut
         constexpr int MAP = decltype(tag)::value;
         if constexpr (MAP != MAP_REC) {
             if (smem > 40 * 1024) {
-                const cudaError_t e = cudaFuncSetAttribute(collide_mma_kernel<MAP, S, DIM>,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                const cudaError_t e = trihost::allow_smem(collide_mma_kernel<MAP, S, DIM>, smem);
                 if (e != cudaSuccess) return e;
             }
             return trihost::launch_behind(collide_mma_kernel<MAP, S, DIM>, g, MMA_THREADS, smem, s, c, rad, n, o, bm);

@@ -75,8 +75,7 @@ cudaError_t launch_one(dim3 g, cudaStream_t s, const float *x, uint32_t n, uint3
     }
     constexpr size_t smem = TileSmem<RHO, R>::bytes(true);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(edm_kernel<MAP, RHO, R, true>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = trihost::allow_smem(edm_kernel<MAP, RHO, R, true>, smem);
         if (e != cudaSuccess) return e;
     }
     edm_kernel<MAP, RHO, R, true><<<g, dim3(RHO, RHO), smem, s>>>(x, n, d, out, bm);

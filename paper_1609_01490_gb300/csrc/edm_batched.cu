@@ -140,11 +140,11 @@ cudaError_t launch_batched_pipe(cudaStream_t s, const float *x_cat, const uint64
     int dev = 0, nsm = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    uint32_t smem_cnt = count + 1;
-    if (smem_cnt > 4096) smem_cnt = 0;  // large batches search the offsets in global memory
+    constexpr uint32_t MOST = 4096;  // larger batches search the offsets in global memory
+    const uint32_t smem_cnt = count < MOST ? count + 1 : 0;
     const size_t dyn = TileSmem<RHO, R>::bytes(PIPE) + (size_t)smem_cnt * sizeof(uint64_t);
-    if (cudaFuncSetAttribute(edm_batched_kernel<RHO, R, PIPE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)dyn) != cudaSuccess)
+    if (trihost::allow_smem(edm_batched_kernel<RHO, R, PIPE>,
+                            TileSmem<RHO, R>::bytes(PIPE) + MOST * sizeof(uint64_t)) != cudaSuccess)
         return cudaErrorInvalidValue;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, edm_batched_kernel<RHO, R, PIPE>, RHO * RHO, dyn);
     if (per < 1) per = 1;

@@ -77,6 +77,11 @@ constexpr uint32_t STATIC_PCT = 80;        // share of the units assigned up fro
 constexpr uint32_t DYN_CHUNK = 2;          // units per grab from the global counter afterwards
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr int MAX_STAGES = 12;             // B ring depth cap (16 KB stages)
+// Dynamic shared memory of the Gram kernel: alignment, norms and scales, barriers, then
+// operand chunks, at most GRAM_SMEM at any d (2 KB of SMEM_LIMIT stay for its variables).
+constexpr int GRAM_FIXED = 1024 + NEPI * NORM_FLOATS * 4 + 8 * (7 + 2 * MAX_STAGES);
+constexpr int GRAM_SMEM = GRAM_FIXED + (SMEM_LIMIT - GRAM_FIXED) / CHUNK_BYTES * CHUNK_BYTES;
+static_assert(GRAM_SMEM <= SMEM_LIMIT - 2048, "room for the kernel's own shared variables");
 
 constexpr float TAU_X3 = 0.0625f;  // flag threshold of TRI_BF16X3 (no bound asked for)
 // A pair with d^2 <= tau (|x_i|^2 + |x_j|^2) + TINY is flagged: below 2^-116 the
@@ -1164,10 +1169,10 @@ bool plan(uint32_t d, int prec, TcPlan &p)
 {
     p.dp = (d + KCH - 1) / KCH * KCH;
     p.nkc = p.dp / KCH;
-    const size_t fixed = 1024 /*align*/ + NEPI * NORM_FLOATS * 4 + 8 * (7 + 2 * MAX_STAGES);
+    const size_t fixed = GRAM_FIXED;
     const size_t a = (size_t)P * p.nkc * CHUNK_BYTES, st = CHUNK_BYTES;  // one row block per CTA
     if (d > (prec == TRI_BF16X6 ? 192u : 320u)) return false;  // the documented limits
-    static_assert(1024 + NEPI * NORM_FLOATS * 4 + 8 * (7 + 2 * MAX_STAGES) + 12 * CHUNK_BYTES <= SMEM_LIMIT,
+    static_assert(GRAM_FIXED + 12 * CHUNK_BYTES <= SMEM_LIMIT,
                   "d = 320 leaves at least two operand stages");
     p.stages = (uint32_t)std::min<size_t>(MAX_STAGES, (SMEM_LIMIT - fixed - a) / st);
     p.smem = fixed + a + p.stages * st;
@@ -1181,7 +1186,7 @@ bool plan(uint32_t d, int prec, TcPlan &p)
 template <int MP>
 cudaError_t launch_gram(const CUtensorMap &tmap, GramArgs g, size_t smem, bool behind, cudaStream_t s)
 {
-    cudaError_t e = cudaFuncSetAttribute(gram_kernel<MP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = trihost::allow_smem(gram_kernel<MP>, GRAM_SMEM);
     if (e != cudaSuccess) return e;
     static std::mutex mu;
     static int cached_dev = -1, cached_pairs = 0;

@@ -6,6 +6,7 @@
 
 #include "../../include/tri.h"
 #include "pdl.cuh"
+#include "tri_internal.h"
 
 namespace {
 
@@ -26,10 +27,13 @@ constexpr int GROUP = 4;  // samples a block takes at a time
 // Floats of shared memory of mlp_pass_kernel: the weights (rows padded by one
 // word, so that neither a row per thread nor a column per thread conflicts) and a
 // group's activations and gradients.
-__host__ __device__ inline uint32_t pass_floats(uint32_t F, uint32_t H1, uint32_t H2)
+__host__ __device__ constexpr uint32_t pass_floats(uint32_t F, uint32_t H1, uint32_t H2)
 {
     return H1 * (F + 1) + H1 + H2 * (H1 + 1) + 2 * H2 + 1 + GROUP * (F + H1 + 2 * H2 + 1);
 }
+
+// The most shapes_ok lets it take.
+constexpr size_t PASS_SMEM = pass_floats(64, 128, 128) * sizeof(float);
 
 // Forward pass and, with BACK, the gradients of the mean squared loss down to z1,
 // in one launch: a block keeps the weights in shared memory and takes the samples
@@ -276,9 +280,7 @@ int pass(const float *theta, const float *X, const float *y, uint32_t B, uint32_
          float *pred, const Batch &w, cudaStream_t s)
 {
     const size_t smem = pass_floats(F, H1, H2) * sizeof(float);
-    if (smem > 48 * 1024 && cudaFuncSetAttribute(mlp_pass_kernel<BACK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem) != cudaSuccess)
-        return TRI_ECUDA;
+    if (smem > 48 * 1024 && trihost::allow_smem(mlp_pass_kernel<BACK>, PASS_SMEM) != cudaSuccess) return TRI_ECUDA;
     // a group of samples per block until the weights are read by 1024 blocks
     const uint32_t groups = (uint32_t)(((uint64_t)B + GROUP - 1) / GROUP);
     mlp_pass_kernel<BACK><<<groups < 1024u ? groups : 1024u, MLP_THREADS, smem, s>>>(layout(theta, F, H1, H2), X, y, B, F,

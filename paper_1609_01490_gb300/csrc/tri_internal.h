@@ -8,6 +8,18 @@
 
 namespace trihost {
 
+// Lets a kernel take up to `most` bytes of dynamic shared memory.  The limit belongs to
+// the kernel and the device, not to a launch, and calls on other threads set it too:
+// `most` is the same in every call, so that none lowers it between another's call
+// and launch.
+template <class K>
+cudaError_t allow_smem(K *kernel, size_t most)
+{
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // reported by the caller's status alone
+    return e;
+}
+
 // FP32 direct-difference EDM under any block map (edm.cu).
 int edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int map, uint32_t rho, uint32_t reg,
              cudaStream_t s);

@@ -269,6 +269,47 @@ def test_life_step_default_tiles(orc, n, rho):
         assert np.array_equal(out.cpu().numpy(), ref), name
 
 
+# ------------------------------------------------------------- host threads --
+def test_calls_of_different_sizes_from_threads():
+    """Kernels that take more shared memory than by default, at sizes that differ from
+    thread to thread: no call lowers the limit under another's launch."""
+    import threading
+
+    import torch
+    t, D = tri(), dev()
+    errors = []
+
+    def forward(F, h1, h2):
+        theta = torch.zeros(h1 * F + h1 + h2 * h1 + 2 * h2 + 1, device=D)
+        X, pred = torch.zeros(8, F, device=D), torch.zeros(8, device=D)
+        ws = torch.empty(t.tri_mlp_workspace_size(8, h1, h2) // 4, device=D)
+        for _ in range(20000):
+            t.tri_mlp_forward(theta, X, pred, h1, h2, ws)
+
+    def distances(d, prec):
+        x, out = torch.randn(200, d, device=D), torch.empty(200 * 201 // 2, device=D)
+        ws = torch.empty(t.tri_edm_workspace_size(200, d, prec), dtype=torch.uint8, device=D)
+        for _ in range(4000):
+            t.tri_edm(x, out, prec=prec, workspace=ws)
+
+    def run(f, *args):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                f(*args)
+        except t.TriError as e:
+            errors.append(str(e))
+
+    jobs = [(forward, 64, 128, 128), (forward, 14, 128, 96), (forward, 14, 128, 96), (distances, 64, t.BF16X6),
+            (distances, 320, t.BF16X3)]
+    threads = [threading.Thread(target=run, args=j) for j in jobs]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    assert not errors
+
+
 # --------------------------------------------------------------- cost model --
 @pytest.mark.parametrize("B,F,H1,H2", [(1, 1, 1, 1), (3, 14, 16, 17), (5, 64, 128, 128), (128, 15, 16, 31), (129, 14, 64, 64),
                                        (1030, 14, 33, 96)])
