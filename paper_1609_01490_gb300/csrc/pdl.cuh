@@ -45,7 +45,9 @@ cudaError_t launch_behind(void (*kernel)(P...), dim3 grid, dim3 block, size_t sm
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();  // the caller's to report, not the next launch's
+    return e;
 }
 
 }  // namespace trihost

@@ -37,6 +37,37 @@ def _run(tmp_path, *sources):
     return subprocess.run([exe], env=env).returncode
 
 
+def test_failed_launch_leaves_no_error(tmp_path):
+    """A launch that fails reports its error and leaves none for the next call that asks
+    the runtime for the last one."""
+    (tmp_path / "launch.cu").write_text('''#include "pdl.cuh"
+#include "tri_internal.h"
+extern "C" int last_error;
+__global__ void nothing(int *p) { (void)p; }
+int main()
+{
+    const cudaError_t e = trihost::launch_behind(nothing, dim3(1), dim3(32), 0, nullptr, (int *)nullptr);
+    if (e != cudaErrorInvalidConfiguration || last_error != 0) return 1;
+    const cudaError_t a = trihost::allow_smem(nothing, 1024);
+    return a == cudaErrorInvalidValue && last_error == 0 ? 0 : 2;
+}
+''')
+    # in front of the runtime's own: both calls fail and leave their error behind
+    (tmp_path / "fakes.cpp").write_text('''extern "C" {
+int last_error = 0;
+int cudaLaunchKernelExC(const void *, const void *, void **) { return last_error = 9; }
+int cudaFuncSetAttribute(const void *, int, int) { return last_error = 1; }
+int cudaGetLastError()
+{
+    const int e = last_error;
+    last_error = 0;
+    return e;
+}
+}
+''')
+    assert _run(tmp_path, tmp_path / "launch.cu", tmp_path / "fakes.cpp") == 0
+
+
 def test_shared_memory_limit_is_one_value(tmp_path):
     """The limit of a kernel's shared memory belongs to the process: calls of different
     sizes all set the same one, so that none lowers it between another thread's call
