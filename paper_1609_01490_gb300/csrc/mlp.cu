@@ -22,34 +22,37 @@ struct Batch {
 };
 
 constexpr int MLP_THREADS = 256;
-constexpr int GROUP = 4;  // samples a block takes at a time
+constexpr uint32_t GROUP = 4, MAX_GROUP = 32;  // samples a block takes at a time
 
 // Floats of shared memory of mlp_pass_kernel: the weights (rows padded by one
 // word, so that neither a row per thread nor a column per thread conflicts) and a
 // group's activations and gradients.
-__host__ __device__ constexpr uint32_t pass_floats(uint32_t F, uint32_t H1, uint32_t H2)
+__host__ __device__ constexpr uint32_t pass_floats(uint32_t F, uint32_t H1, uint32_t H2, uint32_t group)
 {
-    return H1 * (F + 1) + H1 + H2 * (H1 + 1) + 2 * H2 + 1 + GROUP * (F + H1 + 2 * H2 + 1);
+    return H1 * (F + 1) + H1 + H2 * (H1 + 1) + 2 * H2 + 1 + group * (F + H1 + 2 * H2 + 1);
 }
 
-// The most shapes_ok lets it take.
-constexpr size_t PASS_SMEM = pass_floats(64, 128, 128) * sizeof(float);
+// The most shapes_ok lets it take: larger groups belong to narrower layers.
+constexpr size_t PASS_SMEM = pass_floats(64, 128, 128, GROUP) * sizeof(float);
+static_assert(pass_floats(64, 128, 1, GROUP) * sizeof(float) <= PASS_SMEM &&
+                  pass_floats(64, 64, 64, MAX_GROUP) * sizeof(float) <= PASS_SMEM,
+              "a larger group only where the wider layer has at most 64 outputs");
 
 // Forward pass and, with BACK, the gradients of the mean squared loss down to z1,
 // in one launch: a block keeps the weights in shared memory and takes the samples
-// four at a time through all the layers.  The passes are bound by latency (the
+// `group` at a time through all the layers.  The passes are bound by latency (the
 // whole batch of the selector's sweep is 2 Mflop): as ten dependent launches a
 // training step took 113 us at B = 391, H1 = H2 = 64, as three it takes 19.  Each sum runs over
 // its inputs in increasing order.
 template <bool BACK>
 __global__ void __launch_bounds__(MLP_THREADS)
     mlp_pass_kernel(const Layout L, const float *__restrict__ X, const float *__restrict__ y, uint32_t B, uint32_t F,
-                    uint32_t H1, uint32_t H2, float *__restrict__ pred, const Batch w)
+                    uint32_t H1, uint32_t H2, uint32_t group, float *__restrict__ pred, const Batch w)
 {
     extern __shared__ float sm[];
     tri::dependents_may_start();
     float *W1 = sm, *b1 = W1 + H1 * (F + 1), *W2 = b1 + H1, *b2 = W2 + H2 * (H1 + 1), *W3 = b2 + H2, *b3 = W3 + H2;
-    float *x = b3 + 1, *z1 = x + GROUP * F, *z2 = z1 + GROUP * H1, *gz2 = z2 + GROUP * H2, *gout = gz2 + GROUP * H2;
+    float *x = b3 + 1, *z1 = x + group * F, *z2 = z1 + group * H1, *gz2 = z2 + group * H2, *gout = gz2 + group * H2;
     const uint32_t tid = threadIdx.x;
     for (uint32_t t = tid; t < H1 * F; t += MLP_THREADS) W1[t / F * (F + 1) + t % F] = L.W1[t];
     for (uint32_t t = tid; t < H2 * H1; t += MLP_THREADS) W2[t / H1 * (H1 + 1) + t % H1] = L.W2[t];
@@ -59,8 +62,8 @@ __global__ void __launch_bounds__(MLP_THREADS)
         W3[t] = L.W3[t];
     }
     if (tid == 0) *b3 = *L.b3;
-    for (uint64_t s0 = (uint64_t)blockIdx.x * GROUP; s0 < B; s0 += (uint64_t)gridDim.x * GROUP) {
-        const uint32_t m = (uint32_t)(B - s0 < GROUP ? B - s0 : GROUP);
+    for (uint64_t s0 = (uint64_t)blockIdx.x * group; s0 < B; s0 += (uint64_t)gridDim.x * group) {
+        const uint32_t m = (uint32_t)(B - s0 < group ? B - s0 : group);
         for (uint32_t t = tid; t < m * F; t += MLP_THREADS) x[t] = X[s0 * F + t];
         __syncthreads();
         for (uint32_t t = tid; t < m * H1; t += MLP_THREADS) {
@@ -279,12 +282,17 @@ template <bool BACK>
 int pass(const float *theta, const float *X, const float *y, uint32_t B, uint32_t F, uint32_t H1, uint32_t H2,
          float *pred, const Batch &w, cudaStream_t s)
 {
-    const size_t smem = pass_floats(F, H1, H2) * sizeof(float);
+    // four samples a block until 1024 blocks read the weights; then as many as keep
+    // the threads busy in the wider layer (B = 200,000, F = 3, H1 = 8, H2 = 5, forward:
+    // 56 us in fours, 14 so)
+    const uint32_t wide = MLP_THREADS / (H1 > H2 ? H1 : H2), per = (uint32_t)(((uint64_t)B + 1023) / 1024);
+    uint32_t group = wide < per ? wide : per;
+    group = group < GROUP ? GROUP : group > MAX_GROUP ? MAX_GROUP : group;
+    const size_t smem = pass_floats(F, H1, H2, group) * sizeof(float);
     if (smem > 48 * 1024 && trihost::allow_smem(mlp_pass_kernel<BACK>, PASS_SMEM) != cudaSuccess) return TRI_ECUDA;
-    // a group of samples per block until the weights are read by 1024 blocks
-    const uint32_t groups = (uint32_t)(((uint64_t)B + GROUP - 1) / GROUP);
+    const uint32_t groups = (uint32_t)(((uint64_t)B + group - 1) / group);
     mlp_pass_kernel<BACK><<<groups < 1024u ? groups : 1024u, MLP_THREADS, smem, s>>>(layout(theta, F, H1, H2), X, y, B, F,
-                                                                                 H1, H2, pred, w);
+                                                                                 H1, H2, group, pred, w);
     return cudaGetLastError() == cudaSuccess ? TRI_OK : TRI_ECUDA;
 }
 

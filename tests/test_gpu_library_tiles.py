@@ -331,6 +331,27 @@ def test_mlp_shapes(orc, B, F, H1, H2):
     assert np.max(np.abs(grad.cpu().numpy().astype(np.float64) - ref_g)) <= 1e-4 * np.max(np.abs(ref_g))
 
 
+@pytest.mark.parametrize("B", [4096, 4097, 9001, 40000])
+@pytest.mark.parametrize("F,H1,H2", [(3, 8, 5), (14, 32, 17), (14, 64, 64)])
+def test_mlp_large_batches(orc, B, F, H1, H2):
+    # from 4097 samples on narrow layers take more of them to a block, up to 32
+    import torch
+    t, D = tri(), dev()
+    rng = np.random.default_rng(B + F)
+    theta = (rng.normal(size=orc.mlp_nparams(F, H1, H2)) * 0.2).astype(np.float32)
+    X, y = rng.normal(size=(B, F)).astype(np.float32), rng.normal(size=B).astype(np.float32)
+    th, Xd, yd = (torch.from_numpy(a).to(D) for a in (theta, X, y))
+    ws = torch.empty(t.tri_mlp_workspace_size(B, H1, H2) // 4, device=D)
+    pred, loss, grad = torch.full((B,), 9.0, device=D), torch.empty(1, device=D), torch.full_like(th, 9.0)
+    t.tri_mlp_forward(th, Xd, pred, H1, H2, ws)
+    t.tri_mlp_grad(th, Xd, yd, loss, grad, H1, H2, ws)
+    # as in test_mlp_shapes
+    np.testing.assert_allclose(pred.cpu().numpy(), orc.mlp_forward(theta.astype(np.float64), X, H1, H2), rtol=1e-4, atol=1e-5)
+    ref_loss, ref_g = orc.mlp_grad(theta.astype(np.float64), X, y, H1, H2)
+    assert float(loss.item()) == pytest.approx(ref_loss, rel=1e-5)
+    assert np.max(np.abs(grad.cpu().numpy().astype(np.float64) - ref_g)) <= 1e-4 * np.max(np.abs(ref_g))
+
+
 @pytest.mark.parametrize("e", [-45, -27, 0, 56])  # sums of squares below 2^-60, about it, ordinary, above 2^100
 @pytest.mark.parametrize("d", [1, 3, 32, 33, 100])
 def test_tc_edm_recomputed_pairs(d, e):
