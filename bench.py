@@ -551,7 +551,7 @@ def run_suite(args):
             def run():
                 for s in range(100):
                     src, dst = (a, b) if s % 2 == 0 else (b, a)
-                    tri.tri_ca_step(src, dst, n, map=m, rho=rho)
+                    tri.tri_ca_step_tile(src, dst, n, map=m, rho=rho)
             return run
         # 128 x 128 cell tiles (rho = 32) are the fastest; rho = 16 beside them
         t = {nm: graph_ms(life(m, 32), 1) / 100 for nm, m in (("lambda", tri.MAP_LAMBDA), ("bb", tri.MAP_BB),

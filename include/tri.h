@@ -347,15 +347,20 @@ TRI_API int tri_edm_batched_partition(const uint32_t *n_k, uint32_t count, uint3
  *   in, out (device uint8, 16-byte aligned) row-major with leading dimension
  *   ld (bytes); ld >= n and ld a multiple of 16; in != out (no aliasing).
  *   map: LAMBDA, LAMBDA_PDELTA, BB, RB or REC.  rho in {8,16,32}: each block
- *   covers a (4 rho) x (4 rho) cell tile, except that Conway's rule takes 128 x
- *   128-cell tiles from n = 6000 on and other rules 64 x 64 ones at rho = 32 (not
- *   under REC).  Conway's rule runs bit-sliced with
+ *   covers a (4 rho) x (4 rho) cell tile.  The result does not depend on rho, and
+ *   tri_ca_step runs a faster tile where it knows one (not under REC): Conway's
+ *   rule 128 x 128 cells from n = 6000 on, other rules 64 x 64 in place of 128 x
+ *   128.  tri_ca_step_tile is the same step at exactly the tile asked for, to time
+ *   or choose block sizes.  Conway's rule runs bit-sliced with
  *   2 rho threads, each a 32-cell strip of rho/4 consecutive rows held as one
  *   bit per cell (two 16-byte loads per row); other rules run with 4 rho
  *   threads, each a 16-cell strip of byte counters (one 16-byte load per row).
  *   Errors: TRI_EINVAL (null, aliasing, bad ld/rho/map), TRI_ERANGE, TRI_ECUDA.
  */
 TRI_API int tri_ca_step(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld,
+                uint32_t birth_mask, uint32_t survive_mask, int map, uint32_t rho,
+                void *stream);
+TRI_API int tri_ca_step_tile(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld,
                 uint32_t birth_mask, uint32_t survive_mask, int map, uint32_t rho,
                 void *stream);
 
@@ -587,7 +592,8 @@ TRI_API int tri_mlp_argmin(const float *theta, const float *X, uint32_t B, uint3
  * TRI_SELECT_FEATURES features: log2 n, log2 d, log2 rho, log2 of the blocks
  * the map launches, kernel one-hot (EDM, CA, AT), map one-hot (LAMBDA,
  * LAMBDA_PDELTA, BB, RB, REC, UTM), log2 of the tile side (4 rho for EDM
- * and CA, rho for AT).
+ * and CA, rho for AT).  The tiles are those of the calls that the autotuner
+ * times: tri_edm with reg = 4, tri_ca_step_tile, tet_at_energy.
  *
  *   tri_select_features: host only.  Writes the candidates (maps outer, rho
  *     inner) to maps[] / rhos[] and their raw features to X [count][F]

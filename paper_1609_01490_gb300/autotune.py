@@ -11,7 +11,8 @@ against (``selector.py``).
 Kernels and their candidate maps:
   edm: lambda, lambda on P_Delta, BB, RB, REC, UTM (Section 4.2), FP32 direct
        differences, 4 x 4 pairs per thread (reg = 4)
-  ca:  lambda, lambda on P_Delta, BB, RB, REC (one Life step)
+  ca:  lambda, lambda on P_Delta, BB, RB, REC (one Life step at exactly the tile
+       of rho: tri_ca_step_tile)
   at:  tetrahedral lambda, BB (Axilrod-Teller energy)
 REC is skipped where the block count is not a power of two.
 
@@ -47,8 +48,12 @@ def _cache_path() -> str:
     return os.environ.get("TRI_TUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "tri_autotune.json"))
 
 
+# What the cached times of a kernel were taken of: entries of another tile are not read
+_TIMED = {"edm": "edm", "ca": "ca tile", "at": "at"}
+
+
 def _key(kernel: str, n: int, d: int) -> str:
-    return f"{torch.cuda.get_device_name()}|{kernel}|{n}|{d}"
+    return f"{torch.cuda.get_device_name()}|{_TIMED[kernel]}|{n}|{d}"
 
 
 def cand_name(map_id: int, rho: int) -> str:
@@ -89,7 +94,7 @@ class _Workload:
         if self.kernel == "edm":
             tri.tri_edm(self.x, self.out, map=map_id, rho=rho, reg=0)
         elif self.kernel == "ca":
-            tri.tri_ca_step(self.a, self.b, self.n, map=map_id, rho=rho)
+            tri.tri_ca_step_tile(self.a, self.b, self.n, map=map_id, rho=rho)
         else:
             tri.tet_at_energy(self.p, self.e, 1.0, map_id, rho, self.ws)
 

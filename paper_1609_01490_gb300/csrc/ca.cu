@@ -308,7 +308,7 @@ static int ca_args_ok(const uint8_t *in, const uint8_t *out, uint32_t n, size_t 
     return TRI_OK;
 }
 
-// The tile a whole-grid step runs at (the result does not depend on it).  Large
+// The tile that tri_ca_step runs at (the result does not depend on it).  Large
 // grids under Conway's rule take 128 x 128 cells whatever rho: blocks of four
 // warps that prefetch ahead, against one-warp blocks bound by load latency (lambda,
 // rho = 16 / 32: n = 16384 75 / 56 us, 8000 21.6 / 19.0, 6000 12.6 / 12.4, 4096
@@ -328,9 +328,17 @@ extern "C" int tri_ca_step(const uint8_t *in, uint8_t *out, uint32_t n, size_t l
 {
     const int ok = ca_args_ok(in, out, n, ld, birth_mask, survive_mask, rho);
     if (ok != TRI_OK) return ok;
+    rho = step_rho(n, birth_mask | (survive_mask << 9), map, rho);
+    return tri_ca_step_tile(in, out, n, ld, birth_mask, survive_mask, map, rho, stream);
+}
+
+extern "C" int tri_ca_step_tile(const uint8_t *in, uint8_t *out, uint32_t n, size_t ld, uint32_t birth_mask,
+                                uint32_t survive_mask, int map, uint32_t rho, void *stream)
+{
+    const int ok = ca_args_ok(in, out, n, ld, birth_mask, survive_mask, rho);
+    if (ok != TRI_OK) return ok;
     const uint32_t table = birth_mask | (survive_mask << 9);  // bit count + 9*alive
     cudaStream_t s = (cudaStream_t)stream;
-    rho = step_rho(n, table, map, rho);
     const uint32_t S = 4 * rho, m = (n + S - 1) / S;
     BlockMap bm{};
     bm.m = m;

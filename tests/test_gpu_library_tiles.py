@@ -269,6 +269,28 @@ def test_life_step_default_tiles(orc, n, rho):
         assert np.array_equal(out.cpu().numpy(), ref), name
 
 
+@pytest.mark.parametrize("n", [1, 65, 1000, 5999, 6000, 6001])
+@pytest.mark.parametrize("rule", ["life", "highlife"])
+def test_life_step_tiles_agree(orc, n, rule):
+    # both sides of the size from which Conway's rule takes one tile whatever rho, and
+    # every tile asked for by itself
+    import torch
+    t, D = tri(), dev()
+    birth, survive = (t.LIFE_BIRTH, t.LIFE_SURVIVE) if rule == "life" else ((1 << 3) | (1 << 6), (1 << 2) | (1 << 3))
+    ld = -(-n // 16) * 16
+    g = inputs.ca_grid(n, seed=n, ld=ld)
+    if n <= 1000:
+        g[np.triu_indices(n, 1)] = 5
+    a = torch.from_numpy(g).to(D)
+    ref = torch.from_numpy(orc.ca_step(g, birth, survive)).to(D)
+    for rho in (8, 16, 32):
+        for name in ("LAMBDA", "LAMBDA_PDELTA", "BB", "RB"):
+            for call in (t.tri_ca_step, t.tri_ca_step_tile):
+                out = a.clone()
+                call(a, out, n, birth_mask=birth, survive_mask=survive, map=getattr(t, "MAP_" + name), rho=rho)
+                assert torch.equal(out, ref), (rho, name, call.__name__)
+
+
 # ------------------------------------------------------------- host threads --
 def test_calls_of_different_sizes_from_threads():
     """Kernels that take more shared memory than by default, at sizes that differ from
