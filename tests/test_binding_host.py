@@ -13,7 +13,7 @@ def tri():
 
 
 def test_autotuner_times_the_tiles_it_names(tri, monkeypatch):
-    # every candidate runs at its own rho, the Life step at exactly its tile
+    # every candidate runs at its own rho: 4 x 4 pairs per thread, exactly the Life tile
     from paper_1609_01490_gb300 import autotune
     calls = []
     for name in ("tri_edm", "tri_ca_step", "tri_ca_step_tile", "tet_at_energy"):
@@ -26,4 +26,5 @@ def test_autotuner_times_the_tiles_it_names(tri, monkeypatch):
         for rho in autotune.RHOS:
             work.launch(tri.MAP_LAMBDA, rho)
     assert [c[0] for c in calls] == ["tri_edm"] * 3 + ["tri_ca_step_tile"] * 3 + ["tet_at_energy"] * 3
+    assert all(c[2]["reg"] == 4 and c[2]["rho"] == r for c, r in zip(calls[:3], autotune.RHOS))
     assert all(c[2]["rho"] == r for c, r in zip(calls[3:6], autotune.RHOS))
