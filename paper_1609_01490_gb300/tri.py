@@ -123,11 +123,17 @@ def _hptr(t) -> int:
     return t.data_ptr()
 
 
+# The current stream's handle without the Stream object around it: the smallest calls
+# are bound by the host (tri_edm, N = 2048, d = 3: 7.8 us a call with it, 6.2 without).
+# Not a public function of torch: None where a version has no such name.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream) -> int | None:
     if stream is None:
-        # the current stream's handle, without the Stream object around it: the smallest
-        # calls are bound by the host (tri_edm, N = 2048, d = 3: 7.8 us a call with it, 6.2 without)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _raw_stream is None:
+            return torch.cuda.current_stream().cuda_stream
+        return _raw_stream(torch.cuda.current_device())
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
 
 

@@ -1,4 +1,6 @@
 """Host side of the binding and of the autotuner, with fakes in place of the device."""
+import types
+
 import pytest
 
 pytest.importorskip("torch")
@@ -10,6 +12,15 @@ def tri():
     build.build()
     from paper_1609_01490_gb300 import tri as t
     return t
+
+
+def test_stream_without_the_raw_handle(tri, monkeypatch):
+    # a torch without the private function: the public current stream
+    import torch
+    monkeypatch.setattr(tri, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: types.SimpleNamespace(cuda_stream=1234))
+    assert tri._stream(None) == 1234
+    assert tri._stream(7) == 7 and tri._stream(types.SimpleNamespace(cuda_stream=9)) == 9
 
 
 def test_autotuner_times_the_tiles_it_names(tri, monkeypatch):
