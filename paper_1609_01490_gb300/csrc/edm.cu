@@ -114,14 +114,16 @@ int trihost::edm_fp32(const float *x, uint32_t n, uint32_t d, float *out, int ma
         // out of it; REC keeps that tile, whose block rows it needs a power of two of
         const int st = trihost::map_range(map, ((uint64_t)n + 4 * rho - 1) / (4 * rho));
         if (st != TRI_OK) return st;
-        // few features: the row tile once there are several of its blocks per SM
+        // few features: the row tile once there are 800 of its blocks (d <= 4) or 1200,
+        // five and eight for each of 152 SMs; 5 to 7 features take the sums of 8
         // (d = 3, us, 4 x 4 pairs a thread / row tile: n = 65536 1995 / 1209, n = 8000 32.5 /
         // 24.9, n = 5000 14.4 / 14.1, n = 4000 10.1 / 10.6, n = 2048 4.7 / 7.8;
-        // d = 8: n = 7000 36.9 / 32.9, n = 6000 28.7 / 28.2, n = 5000 20.6 / 22.6)
+        // d = 8: n = 7000 36.9 / 32.9, n = 6000 28.7 / 28.2, n = 5000 20.6 / 22.6; d = 5:
+        // n = 6144 / 6145 23.5 / 23.6, and with the staging before that 8000 43.4 / 34.9)
         if (d <= (uint32_t)rows::MAX_D && T2(((uint64_t)n + rows::S - 1) / rows::S) >= (d <= 4 ? 800u : 1200u))
             return launch_rows(x, n, d, out, map, s);
         // more features: 8 x 8 pairs per thread, bound by arithmetic with half the
-        // shared-memory reads per pair, once there are three blocks per SM (4 x 4 / 8 x
+        // shared-memory reads per pair, once there are 500 of its blocks (4 x 4 / 8 x
         // 8 at rho = 16, us: n = 20011 d = 100 1627 / 1318, d = 32 616 / 488, d = 9 293 /
         // 238; d = 64 n = 4000 49 / 47, n = 2500 24.4 / 26.9)
         const uint64_t m8 = ((uint64_t)n + 8 * rho - 1) / (8 * rho);

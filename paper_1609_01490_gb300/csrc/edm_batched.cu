@@ -179,7 +179,12 @@ extern "C" int tri_edm_batched(const float *x_cat, const uint64_t *pt_off, const
     if (!x_cat || !pt_off || !n_k || !out_cat || !out_off || !workspace || d == 0 || count == 0)
         return TRI_EINVAL;
     if (!trihost::rho_ok(rho)) return TRI_EINVAL;
-    if (reg == 0) reg = 4;  // 4 x 4 pairs per thread: fastest at every d measured (3, 64, 128)
+    // reg = 0: 4 x 4 pairs per thread.  Better for small instances, where 8 x 8 tiles
+    // overhang, at any d; 8 x 8 at rho = 16 is for large ones, and the autotuner finds it
+    // (us, 4 x 4 / 8 x 8 at rho = 16: 10 instances up to 512 points, d = 64 17.8 / 29.8; 100
+    // up to 1000, d = 3 25.8 / 30.6, d = 64 66.9 / 73.1; 300 up to 4000, d = 3 390 / 350, d =
+    // 64 1580 / 1368).
+    if (reg == 0) reg = 4;
     // 8 x 8 pairs per thread only with rho <= 16 (registers and shared memory)
     if ((reg != 1 && reg != 2 && reg != 4 && reg != 8) || (reg == 8 && rho > 16)) return TRI_EINVAL;
     size_t need = 0;

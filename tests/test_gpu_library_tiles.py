@@ -178,6 +178,25 @@ def test_edm_row_tiles_at_chosen_sizes(d, n):
             assert bool((buf[:8 + off] == -7.0).all()) and bool((buf[8 + off + size:] == -7.0).all())
 
 
+@pytest.mark.parametrize("d,sizes", [(1, (4993, 5119, 5120)), (2, (4993,)), (3, (4993, 5119, 5120)), (4, (5121,)),
+                                     (5, (6145,)), (6, (6271,)), (7, (6272,)), (8, (6145, 6273))])
+def test_edm_row_tiles_under_every_map(d, sizes):
+    # the smallest sizes that take the row tile, one row more or less in its last tile row
+    import torch
+    t, D = tri(), dev()
+    for n in sizes:
+        x = torch.from_numpy(inputs.edm_normal_points(n, d, seed=n + d)).to(D)
+        size = n * (n + 1) // 2
+        ref = torch.empty(size, device=D)
+        t.tri_edm(x, ref, reg=4)
+        for k, name in enumerate(("LAMBDA", "LAMBDA_PDELTA", "BB", "RB")):
+            off = (n + k) % 4
+            buf = torch.full((size + 16,), -7.0, device=D)
+            t.tri_edm(x, buf[8 + off:8 + off + size], map=getattr(t, "MAP_" + name))
+            assert torch.equal(buf[8 + off:8 + off + size], ref), (n, name)
+            assert bool((buf[:8 + off] == -7.0).all()) and bool((buf[8 + off + size:] == -7.0).all())
+
+
 @pytest.mark.parametrize("d", [9, 16, 33, 100])
 def test_edm_chosen_square_tiles(d):
     # sizes on both sides of the choice between 4 x 4 and 8 x 8 pairs per thread
