@@ -782,7 +782,7 @@ def run_split(args, rank: int, world: int, local: int):
     cfg["parallelism"] = f"one triangle split in {world} row bands of equal pair count (tri_edm_partition)"
     line = {"metric": "pairs/s", "value": P / (ms * 1e-3), "unit": "pairs/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "strong",
-            "vs_baseline": None, "dtype": "bf16", "data": "synthetic", "config": cfg, "clocks": clocks,
+            "vs_baseline": None, "dtype": "fp16", "data": "synthetic", "config": cfg, "clocks": clocks,
             "gpu_launches": args.steps * 3, "band": {"rows": [rb, re_], "pairs": pe - pb}}
     if e2e:
         line["e2e"] = e2e
@@ -1082,7 +1082,7 @@ def main():
     line = {
         "metric": "pairs/s", "value": value, "unit": "pairs/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": {"fp32": "f32", "bf16x3": "bf16", "bf16x6": "bf16"}[args.prec],
+        "vs_baseline": None, "dtype": {"fp32": "f32", "bf16x3": "fp16", "bf16x6": "fp16"}[args.prec],
         "data": "synthetic",
         "config": headline_config(args.prec),
         "bb": {"ms_per_step": ms_bb, "value": job_rate(world, P, ms_bb), "I_bb_over_lambda": ms_bb / ms_step},

@@ -22,7 +22,8 @@
 // lanes per clock and SM; ncu counts 11.7 ALU operations per word and step and
 // the pipe 84% busy at n = 16384.
 // 100 steps at n = 16384: 977 -> 500 us (bytes between passes of 16 steps and
-// column-order words before), at n = 2000: 180 -> 66 us.  256 x 256-cell regions
+// column-order words before), 469 with the passes launched behind one another; at n =
+// 2000: 180 -> 66 us.  256 x 256-cell regions
 // (8 words, 8 rows a lane) took 514 us: fewer halo cells, but a step's code no
 // longer fits the instruction cache and the last wave runs nearly empty.
 #include <cuda_runtime.h>

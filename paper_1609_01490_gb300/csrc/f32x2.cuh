@@ -1,6 +1,9 @@
 // Two FP32 lanes per instruction: the packed add/sub/mul/fma of sm_100 and
-// later on .b64 register pairs, each lane rounded to nearest exactly as the
-// scalar FP32 instruction would round it.
+// later on .b64 register pairs, each lane rounded to nearest as the scalar FP32
+// instruction would round it.  A product whose only use is a packed sum or
+// difference is not safe from fusion: ptxas makes one multiply-add of the two, .rn or
+// not (x x - RN(x x) comes out as the product's rounding error).  Where the separate
+// roundings matter, the scalar __fmul_rn and __fadd_rn keep them.
 #pragma once
 
 namespace tri {
